@@ -240,7 +240,8 @@ def run_reference(args, rank):
 # -- traffic recorded from an ncu capture of the current kernel source ----------
 
 # the sources the profiled compress kernel is compiled from
-KERNEL_SOURCES = ("kernels.cu", "kernels.cuh", "compress_fast.cuh", "codec.cuh", "common.cuh",
+KERNEL_SOURCES = ("kernels.cu", "kernels.cuh", "compress_cta.cuh", "lz4_cta.cuh",
+                  "shuffle_cta.cuh", "compress_fast.cuh", "codec.cuh", "common.cuh",
                   "lz4_warp.cuh", "shuffle.cuh")
 
 
@@ -1422,7 +1423,7 @@ def main():
     if inst:
         peak_i = issue_peak_ginst(clk.get("sm_mhz"))
         ach_i = inst / (comp_avg_ms / 1e3) / 1e9
-        issue_line = {"bound": "issue", "kernel": "compress_fast_kernel", "achieved": ach_i,
+        issue_line = {"bound": "issue", "kernel": "compress_cta_kernel", "achieved": ach_i,
                       "peak": peak_i, "unit": "G warp-instructions/s", "frac": ach_i / peak_i,
                       "inst_per_launch": inst}
 
@@ -1442,7 +1443,7 @@ def main():
                       "decompress": {"mean": dec_avg_ms, "median": statistics.median(dec_ms),
                                      "best": min(dec_ms)}},
         "ratio": slen / nbytes,
-        "roofline": {"bound": "hbm", "kernel": "compress_fast_kernel (fused round+shuffle+LZ4)",
+        "roofline": {"bound": "hbm", "kernel": "compress_cta_kernel (fused round+shuffle+LZ4)",
                      "achieved": achieved, "peak": hbm, "peak_kind": peak_kind, "unit": "GB/s",
                      "frac": achieved / hbm, "traffic": traffic,
                      "algorithmic_bytes": alg_c},

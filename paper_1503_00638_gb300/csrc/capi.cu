@@ -90,6 +90,8 @@ uint32_t persistent_grid(uint32_t smem_per_cta, uint64_t work)
 struct WsLayout {
     size_t state, autos, pairs, cft, qtab, offsets, segs, slots, gslots, total;
     uint32_t gslot_warps;  // warps the general compressor's slots cover
+    size_t cslots;         // staging slots of the level-0 compressor (the same space)
+    uint32_t cslot_ctas;   // CTAs they cover
 };
 
 // SMs the general compressor's staging slots are sized for (at least the
@@ -116,8 +118,8 @@ VisOpts vis_opts(int flags, int64_t n_freq, int64_t n_in, int64_t n_time)
     return o;
 }
 
-// Whether compress takes the fast kernel: full blocks of at most 8 KiB of 2-,
-// 4- or 8-byte elements (a cube in any order, any time axis).
+// Whether level-1 compress takes the fast kernel: full blocks of at most 8 KiB
+// of 2-, 4- or 8-byte elements (a cube in any order, any time axis).
 bool fast_shape(const Geometry &g)
 {
     return shuffle_inplace_ok(g.es, g.B);
@@ -132,6 +134,7 @@ WsLayout ws_layout(int op, const Geometry &g, size_t n_auto, size_t n_prod, uint
     if (op == BSGPU_OP_COMPRESS || op == BSGPU_OP_COMPRESS_VIS) {
         L.state = o;
         o += r256((size_t)g.nb * 8);
+        const size_t slots0 = o;
         if (g.nb && fast_shape(g)) {
             L.slots = o;
             o += (size_t)FAST_MAX_WARPS * 2 * FAST_SLOT_BYTES;
@@ -150,6 +153,16 @@ WsLayout ws_layout(int op, const Geometry &g, size_t n_auto, size_t n_prod, uint
             L.gslots = o;
             L.gslot_warps = (uint32_t)w;
             o += r256((size_t)w * 2 * compress_slot_bytes(maxb));
+        }
+        // the level-0 compressor's slots take the place of the other two's
+        // (a call uses one or the other)
+        if (g.nb && compress_cta_ok(g.es, g.B)) {
+            uint64_t ctas = compress_cta_max(g.B * g.es, GEN_MAX_SMS);
+            if (ctas > g.nb) ctas = g.nb;
+            L.cslots = slots0;
+            L.cslot_ctas = (uint32_t)ctas;
+            const size_t end = slots0 + r256(compress_cta_slots_bytes(g.B * g.es, L.cslot_ctas));
+            if (o < end) o = end;
         }
     }
     if (op == BSGPU_OP_COMPRESS_VIS || op == BSGPU_OP_REDUCE_PRECISION) {
@@ -451,7 +464,11 @@ static int compress_common(const void *in, const Geometry &g, int level, void *o
     if (cudaMemsetAsync(ws, 0, L.state + (size_t)g.nb * 8, s) != cudaSuccess)
         return BSGPU_ERR_CUDA;
     if (g.nb == 0) return cuda_err(launch_compress_small(a, s));
-    // full blocks through the fast kernel when its slots are in the
+    if (level == 0 && L.cslots) {
+        a.slots = reinterpret_cast<uint8_t *>(ws) + L.cslots;
+        return cuda_err(launch_compress_cta(a, L.cslot_ctas, s));
+    }
+    // level 1: full blocks through the fast kernel when its slots are in the
     // workspace, the rest (a shortened last block, other shapes) through the
     // general one; both place blocks through the same look-back state
     const uint32_t nfull = g.nb - (g.last_B != g.B ? 1u : 0u);
@@ -463,9 +480,9 @@ static int compress_common(const void *in, const Geometry &g, int level, void *o
         const bool ts = vis && vis->tslow;
         // 4-byte components of a cube whose time axis is not a multiple of 16
         const bool ps = vis && !vis->tslow && g.es == 4 && (vis->T % 16u) != 0;
-        uint64_t grid = (uint64_t)sms * (ts ? compress_fast_tslow_blocks_per_sm(level, g.es)
-                                            : ps ? compress_fast_ps_blocks_per_sm(level)
-                                                 : compress_fast_blocks_per_sm(level, g.es));
+        uint64_t grid = (uint64_t)sms * (ts ? compress_fast_tslow_blocks_per_sm(g.es)
+                                            : ps ? compress_fast_ps_blocks_per_sm()
+                                                 : compress_fast_blocks_per_sm(g.es));
         if (grid > nfull) grid = nfull;
         if (grid > FAST_MAX_WARPS) grid = FAST_MAX_WARPS;
         CodecArgs f = a;

@@ -492,6 +492,33 @@ BSG_D void compress_prepare(const CodecArgs &a, uint32_t tile, uint8_t *in, uint
     shuffle_block(in, tmp, Bb, a.es, lane);
 }
 
+// What follows the last block, which ends at stream offset `end`: the (n mod
+// 8) trailing elements verbatim and the stream length.  One warp.
+BSG_D void compress_place_end(const CodecArgs &a, uint64_t end, uint32_t lane)
+{
+    const uint64_t first = a.n_elem - a.tail_elems;
+    const uint32_t tb = a.tail_elems * a.es;
+    if (end + tb > a.out_cap) {
+        if (lane == 0) set_status(a.status, BSGPU_ERR_SPACE);
+        return;
+    }
+    if (a.vis.enabled) {
+        // the tail as 32-bit components, each rounded like any other
+        const uint32_t tc = tb / 4;
+        const uint64_t c0 = first * a.es / 4;
+        if (lane < tc) {
+            const uint32_t *src = reinterpret_cast<const uint32_t *>(a.in);
+            const uint64_t fi = c0 + lane;
+            const uint32_t x = src[2 * vis_src(a.vis, fi >> 1) + (fi & 1)];
+            const uint32_t u = reduce_component_at(x, fi, a.vis);
+            for (int k = 0; k < 4; k++) a.out[end + 4 * lane + k] = (uint8_t)(u >> (8 * k));
+        }
+    } else {
+        for (uint32_t k = lane; k < tb; k += 32) a.out[end + k] = a.in[first * a.es + k];
+    }
+    if (lane == 0) *a.out_bytes = end + tb;
+}
+
 // Write block `tile` (its 4-byte length field and cs LZ4 bytes at `blk`, in
 // shared or global memory) at stream offset D, with the index entry, the
 // chunk header (block 0) and, after the last block, the verbatim tail.
@@ -505,31 +532,7 @@ BSG_D void compress_place(const CodecArgs &a, uint32_t tile, const uint8_t *blk,
     copy_out(blk, a.out + D, 4 + cs, lane);
     if (a.block_offsets && lane == 0) a.block_offsets[tile] = D;
     if (tile == 0) write_chunk_header(a.out, a.n_elem * a.es, a.B * a.es, lane);
-    if (tile + 1 == a.nb) {
-        // the (n mod 8) trailing elements follow the last block verbatim
-        const uint64_t end = D + 4 + cs;
-        const uint64_t first = a.n_elem - a.tail_elems;
-        const uint32_t tb = a.tail_elems * a.es;
-        if (end + tb > a.out_cap) {
-            if (lane == 0) set_status(a.status, BSGPU_ERR_SPACE);
-            return;
-        }
-        if (a.vis.enabled) {
-            // the tail as 32-bit components, each rounded like any other
-            const uint32_t tc = tb / 4;
-            const uint64_t c0 = first * a.es / 4;
-            if (lane < tc) {
-                const uint32_t *src = reinterpret_cast<const uint32_t *>(a.in);
-                const uint64_t fi = c0 + lane;
-                const uint32_t x = src[2 * vis_src(a.vis, fi >> 1) + (fi & 1)];
-                const uint32_t u = reduce_component_at(x, fi, a.vis);
-                for (int k = 0; k < 4; k++) a.out[end + 4 * lane + k] = (uint8_t)(u >> (8 * k));
-            }
-        } else {
-            for (uint32_t k = lane; k < tb; k += 32) a.out[end + k] = a.in[first * a.es + k];
-        }
-        if (lane == 0) *a.out_bytes = end + tb;
-    }
+    if (tile + 1 == a.nb) compress_place_end(a, D + 4 + cs, lane);
 }
 
 // Drop the L2 lines of a placed block's staging slot without writing them

@@ -151,13 +151,13 @@ BSG_HD int32_t round_int_pow2(int32_t x, int k)
 {
     if (k <= 0) return x;
     if (k >= 32) return 0;  // |x| <= 2^31 <= g / 2: the nearest (even) multiple is 0
-    const int64_t g = (int64_t)1 << k;
-    int64_t m = (int64_t)x >> k;  // floor
-    const int64_t r = (int64_t)x - m * g, h = g >> 1;
-    if (r > h || (r == h && (m & 1))) m++;
-    int64_t y = m * g;
-    if (y > INT32_MAX) y -= g;
-    return (int32_t)y;
+    // half a granularity, less one where the lower multiple is even, carries
+    // into the kept bits exactly when the upper multiple is nearer (or even)
+    const uint32_t g = 1u << k, odd = ((uint32_t)x >> k) & 1u;
+    const uint32_t sum = (uint32_t)x + ((g >> 1) - 1u) + odd;
+    // a carry into the sign is the multiple 2^31: the one below it instead
+    const uint32_t y = x >= 0 && (int32_t)sum < 0 ? (uint32_t)x : sum;
+    return (int32_t)(y & ~(g - 1u));
 }
 
 // Division by an invariant 32-bit divisor d >= 1 through a multiply-high:

@@ -1,0 +1,507 @@
+// The level-0 compress kernel: [gather ->] round -> bit-transpose -> LZ4 ->
+// placement of one block per CTA step (Sec. 4.2.1, Sec. 6 steps 1-5), for
+// every element size, every block size up to 64 KiB whose bit-rows are whole
+// words (cta_shape_ok), and the shortened last block of such a stream.
+#pragma once
+
+#include "codec.cuh"
+#include "lz4_cta.cuh"
+#include "shuffle_cta.cuh"
+
+namespace bsg {
+
+// How a block's elements are prepared before the transpose.
+enum CtaMode {
+    CTA_PLAIN,    // as they are
+    CTA_GROUP,    // float32 cube, constant c, time axis a multiple of 16: in
+                  // registers, a thread's 32 words being 16 samples of one product
+    CTA_GROUP_X,  // the same for int32, the compensated c or the full-covariance q
+    CTA_SAMPLE    // any time axis and 8-byte samples: in shared memory first
+};
+
+// Resident warps per SM of the kernels with a fixed block size: 28 at 72
+// registers a thread.
+constexpr uint32_t CTA_WARPS_PER_SM = 28;
+
+// Full blocks from which a stream with a shortened last block takes two launches.
+constexpr uint32_t CTA_SPLIT_BLOCKS = 4096;
+
+struct CtaPlan {
+    uint32_t W;          // warps
+    uint32_t tmp;        // bytes of the block buffer
+    uint32_t smem;       // dynamic shared memory
+    uint32_t slot;       // bytes of a staging slot
+};
+__host__ __device__ constexpr CtaPlan cta_plan(uint32_t S)
+{
+    const uint32_t W = cta_warps(S), tmp = r16(S + 16u);
+    return CtaPlan{W, tmp, tmp + r16(cta_scratch_bytes(W)) + 16u, r16(4u + lz4b(S) + 32u)};
+}
+
+// Round 16 complex samples in registers (v[m] = component (m + 4 rot) mod 32
+// of the group) with the constant c.  Per component two additions, the sign
+// and one OR: whether |x| was below 2^(k+23) (and a number) is not tested
+// component by component but once per group, from the exponents of the
+// sums |x| + 2^(k+23), which then all equal that of 2^(k+23).  Returns false
+// when some component needs the full rule (values beyond 2^(k+23), NaN,
+// infinities, an unusable q): the registers are then garbage and the caller
+// rounds the group sample by sample.
+BSG_D bool cta_round_group(const VisParams &P, uint32_t (&v)[32], uint32_t rot, const float *ai,
+                           const float *aj, bool is_auto)
+{
+    const float cc = is_auto ? P.c2 : P.c;
+    uint32_t big = 0, worst = 0;
+#pragma unroll
+    for (int k = 0; k < 8; k++) {
+        const uint32_t c = (k + rot) & 7u;  // samples 2 c and 2 c + 1
+        const float2 Ai = __ldg(reinterpret_cast<const float2 *>(ai + 2 * c));
+        const float2 Aj = __ldg(reinterpret_cast<const float2 *>(aj + 2 * c));
+#pragma unroll
+        for (int s = 0; s < 2; s++) {
+            const uint32_t Q = __float_as_uint(
+                __fmul_rn(__fmul_rn(cc, s ? Ai.y : Ai.x), s ? Aj.y : Aj.x));
+            // magic_bits(Q), the constant 86 << 23 folded in before the shift
+            const uint32_t Tb = ((Q + 0x007fffffu + (86u << 24)) >> 1) & 0x7f800000u;
+            const float T = __uint_as_float(Tb);
+            const uint32_t u = Q - 0x00800000u;   // q_usable: below 0x7f000000
+            worst = worst > u ? worst : u;
+#pragma unroll
+            for (int h = 0; h < 2; h++) {
+                if (h && is_auto) continue;   // the imaginary part of an auto stays
+                uint32_t &w = v[4 * k + 2 * s + h];
+                const float t = __fadd_rn(fabsf(__uint_as_float(w)), T);
+                big |= __float_as_uint(t) ^ Tb;
+                w = __float_as_uint(__fsub_rn(t, T)) | (w & 0x80000000u);
+            }
+        }
+    }
+    return (big & 0x7f800000u) == 0u && worst < 0x7f000000u;
+}
+
+template <int ES, int MODE>
+struct CtaRound {
+    const VisParams *P;
+    uint8_t *buf;
+    uint32_t c_blk;   // complex index of the block's first sample
+    BSG_D void operator()(uint32_t g, uint32_t (&v)[32]) const
+    {
+        if (MODE == CTA_GROUP_X) {
+            const VisGroupRound<true> round{P, c_blk};
+            round(g, v);
+        } else if (MODE == CTA_GROUP) {
+            const uint32_t cg = c_blk + 16u * g;
+            const uint32_t fp = fastdiv(cg, P->dT), t0 = cg - fp * P->T;
+            const uint32_t f = fastdiv(fp, P->dP), p = fp - f * P->P;
+            const uint32_t ij = __ldg(P->pairs + p), i = ij & 0xffffu, j = ij >> 16;
+            const float *ai = P->autos + (size_t)(f * P->n_in + i) * P->T + t0;
+            const float *aj = P->autos + (size_t)(f * P->n_in + j) * P->T + t0;
+            if (!cta_round_group(*P, v, g & 7u, ai, aj, i == j)) {
+                // rare: the group's samples again from shared memory, by the full rule
+                uint4 *grp = reinterpret_cast<uint4 *>(buf + 128u * g);
+                const float cc = i == j ? P->c2 : P->c;
+#pragma unroll 1
+                for (uint32_t c = 0; c < 16; c++) {
+                    const float q = __fmul_rn(__fmul_rn(cc, __ldg(ai + c)), __ldg(aj + c));
+                    float *x = reinterpret_cast<float *>(grp) + 2u * c;
+                    x[0] = reduce_one(x[0], q);
+                    if (i != j) x[1] = reduce_one(x[1], q);
+                }
+#pragma unroll
+                for (uint32_t k = 0; k < 8; k++) {
+                    const uint4 q = grp[(k + g) & 7u];
+                    v[4 * k] = q.x;
+                    v[4 * k + 1] = q.y;
+                    v[4 * k + 2] = q.z;
+                    v[4 * k + 3] = q.w;
+                }
+            }
+        }
+    }
+};
+
+// Start loading block `tile` (bytes long) into buf; true when a bulk copy is
+// in flight on `bar`.  The ragged end (< 16 bytes, a shortened last block)
+// comes by plain loads.
+BSG_D bool cta_load(uint8_t *buf, const uint8_t *src, uint32_t bytes, uint64_t *bar)
+{
+    const uint32_t bulk = bytes & ~15u;
+    if (threadIdx.x == 0 && bulk) {
+        mbar_arrive_expect_tx(bar, bulk);
+        bulk_g2s(buf, src, bulk, bar);
+    }
+    if (threadIdx.x < (bytes & 15u)) buf[bulk + threadIdx.x] = src[bulk + threadIdx.x];
+    return bulk != 0u;
+}
+
+// Samples c0 .. c0 + n - 1 of a time-slowest cube into time-fastest order.  A
+// block holds n / T series, whose samples of one time are neighbours in the
+// input: consecutive threads take consecutive series, so a request reads
+// whole sectors.  Time axes longer than half a block go sample by sample.
+// With a time axis of whole 16-sample groups the group form below is used.
+BSG_D void cta_gather_samples(const CodecArgs &a, uint8_t *buf, uint32_t c0, uint32_t n)
+{
+    const VisParams &P = a.vis;
+    const uint2 *src = reinterpret_cast<const uint2 *>(a.in);
+    uint2 *d = reinterpret_cast<uint2 *>(buf);
+    const uint32_t tid = threadIdx.x, NT = blockDim.x;
+    if (2u * P.T > n) {
+#pragma unroll 1
+        for (uint32_t k = tid; k < n; k += NT) {
+            const uint32_t c = c0 + k, s = fastdiv(c, P.dT), t = c - s * P.T;
+            d[k] = __ldg(src + (uint64_t)t * P.FP + s);
+        }
+        return;
+    }
+    const uint32_t s0 = fastdiv(c0, P.dT), ns = fastdiv(c0 + n - 1u, P.dT) - s0 + 1u;
+    const uint32_t dt = NT / ns, ds = NT - dt * ns;
+    uint32_t t = tid / ns, s = tid - t * ns;
+    const uint32_t lead = c0 - s0 * P.T;   // samples of the first series before the block
+#pragma unroll 2
+    for (uint32_t it = tid; it < P.T * ns; it += NT) {
+        const uint32_t k = s * P.T + t - lead;   // wraps below zero for t < lead in series 0
+        if (k < n) d[k] = __ldg(src + (uint64_t)t * P.FP + s0 + s);
+        t += dt;
+        s += ds;
+        if (s >= ns) {
+            s -= ns;
+            t++;
+        }
+    }
+}
+
+// A time axis that is a multiple of 16: thread q takes 16-sample series
+// groups q, q + NT, ... (neighbouring threads, neighbouring series), their
+// 16-byte chunks in an order rotated by lane / 4 for whole sectors and
+// distinct banks (as gather_tslow_block).
+BSG_D void cta_gather_groups(const CodecArgs &a, uint8_t *buf, uint32_t c0, uint32_t n)
+{
+    const VisParams &P = a.vis;
+    const uint64_t row = P.FP;
+    const uint2 *src = reinterpret_cast<const uint2 *>(a.in);
+    const uint32_t m = (threadIdx.x >> 2) & 7u;
+#pragma unroll 1
+    for (uint32_t q = threadIdx.x; q < n / 16u; q += blockDim.x) {
+        const uint32_t c = c0 + 16u * q, s = fastdiv(c, P.dT), t0 = c - s * P.T;
+        const uint2 *p = src + (uint64_t)t0 * row + s;
+        uint4 *d = reinterpret_cast<uint4 *>(buf + (size_t)128 * q);
+#pragma unroll
+        for (uint32_t k = 0; k < 8; k++) {
+            const uint32_t x = (k + m) & 7u;
+            const uint2 u = __ldg(p + (uint64_t)(2 * x) * row);
+            const uint2 v = __ldg(p + (uint64_t)(2 * x + 1) * row);
+            d[x] = make_uint4(u.x, u.y, v.x, v.y);
+        }
+    }
+}
+
+// Round n samples from complex index c0 in shared memory, two at a time when
+// the time axis is even (c0 and n then are).
+BSG_D void cta_round_samples(uint8_t *buf, uint32_t c0, uint32_t n, const VisParams &P)
+{
+    const uint32_t tid = threadIdx.x, NT = blockDim.x;
+    if ((P.T & 1u) == 0) {
+        uint4 *b4 = reinterpret_cast<uint4 *>(buf);
+#pragma unroll 1
+        for (uint32_t k = tid; k < n / 2u; k += NT) {
+            const uint32_t c = c0 + 2u * k;
+            const uint32_t fp = fastdiv(c, P.dT), t = c - fp * P.T;
+            const uint32_t f = fastdiv(fp, P.dP), p = fp - f * P.P;
+            b4[k] = reduce_pair(b4[k], __ldg(P.pairs + p), f, t, P);
+        }
+    } else {
+        uint2 *b2 = reinterpret_cast<uint2 *>(buf);
+#pragma unroll 1
+        for (uint32_t k = tid; k < n; k += NT) {
+            const uint32_t c = c0 + k;
+            const uint32_t fp = fastdiv(c, P.dT), t = c - fp * P.T;
+            const uint32_t f = fastdiv(fp, P.dP), p = fp - f * P.P;
+            b2[k] = reduce_sample(b2[k], __ldg(P.pairs + p), f, t, P);
+        }
+    }
+}
+
+// Copy len bytes from 16-byte aligned global `s` (a staging slot, in L2) to
+// global `g` (any alignment), as copy_out does from shared memory.  (Two to
+// four chunks per thread in flight: no faster, the registers cost as much.)
+BSG_D void cta_copy_out(const uint8_t *s, uint8_t *g, uint32_t len)
+{
+    const uint32_t tid = fresh_tid(), NT = blockDim.x;
+    uint32_t head = (uint32_t)((16u - ((uintptr_t)g & 15u)) & 15u);
+    if (head > len) head = len;
+    if (tid < head) g[tid] = __ldcg(s + tid);
+    const uint32_t nchunk = (len - head) / 16u;
+    const uint4 *s4 = reinterpret_cast<const uint4 *>(s);
+    const uint32_t q = (head >> 2) & 3u, sh = (head & 3u) * 8u;
+#pragma unroll 1
+    for (uint32_t c = tid; c < nchunk; c += NT) {
+        const uint32_t so = head + 16u * c;
+        const uint4 A = __ldcg(s4 + (so >> 4)), B = __ldcg(s4 + (so >> 4) + 1);
+        // the five words from word q of A on, moved down by whole words first
+        uint32_t w0 = A.x, w1 = A.y, w2 = A.z, w3 = A.w, w4 = B.x;
+        if (q & 1u) {
+            w0 = w1; w1 = w2; w2 = w3; w3 = w4; w4 = B.y;
+        }
+        if (q & 2u) {
+            w0 = w2; w1 = w3; w2 = w4; w3 = (q & 1u) ? B.z : B.y; w4 = (q & 1u) ? B.w : B.z;
+        }
+        *reinterpret_cast<uint4 *>(g + so) =
+            make_uint4(funnel_r(w0, w1, sh), funnel_r(w1, w2, sh), funnel_r(w2, w3, sh),
+                       funnel_r(w3, w4, sh));
+    }
+    const uint32_t k = head + 16u * nchunk + tid;
+    if (k < len) g[k] = __ldcg(s + k);
+}
+
+// Block `tile` from its staging slot (4 + cs bytes) to stream offset D, with
+// its index entry.
+BSG_D void cta_place(const CodecArgs &a, uint32_t tile, const uint8_t *slot, uint32_t cs, uint64_t D)
+{
+    if (D + 4 + cs > a.out_cap) {
+        if (threadIdx.x == 0) set_status(a.status, BSGPU_ERR_SPACE);
+        return;
+    }
+    cta_copy_out(slot, a.out + D, 4 + cs);
+    if (a.block_offsets && threadIdx.x == 0) a.block_offsets[tile] = D;
+}
+
+// Exclusive prefix of a block whose size is published, as lookback_resolve,
+// but at most `looks` looks in vain: LB_UNKNOWN then.  (Looking at 64, 128 or
+// 256 predecessors per step instead of 32 changed nothing: 224-234 us on the
+// 33024 blocks below; sums of groups of 128 blocks by atomics, which thousands
+// of warps read, kept the atomics waiting: 268 to 970 us.)
+constexpr uint64_t LB_UNKNOWN = ~0ull;
+
+BSG_D uint64_t lookback_some(uint64_t *state, uint32_t tile, uint64_t agg, uint32_t looks,
+                             uint32_t lane)
+{
+    uint64_t excl = 0;
+    uint32_t spins = 0;
+    int64_t base = (int64_t)tile - 1;   // blocks base, base - 1, ... are still to be added
+    for (bool done = tile == 0; !done;) {
+        const int64_t idx = base - (int64_t)lane;
+        const uint64_t v = idx >= 0 ? ld_relaxed_u64(state + idx) : LB_FP;
+        const uint32_t flag = (uint32_t)(v >> 62);
+        const uint32_t pm = __ballot_sync(FULL, flag == 2), im = __ballot_sync(FULL, flag == 0);
+        const uint32_t first = pm ? (uint32_t)(__ffs(pm) - 1) : 32u;
+        if (im & (first >= 32u ? FULL : (1u << first) - 1u)) {
+            if (++spins >= looks) return LB_UNKNOWN;
+            if (spins > 4096) __nanosleep(100);
+            continue;
+        }
+        // the sizes of 32 blocks add up to less than 2^32
+        excl += __reduce_add_sync(FULL, lane < first ? (uint32_t)v : 0u);
+        if (pm) {
+            excl += __shfl_sync(FULL, v, first) & LB_VM;
+            done = true;
+        }
+        base -= 32;
+    }
+    if (tile && lane == 0) st_relaxed_u64(state + tile, LB_FP | (excl + agg));
+    return excl;
+}
+
+// One block at a time per CTA (persistent, tiles in order from a counter):
+// the block is transposed in place through registers and encoded into a
+// staging slot in global memory (it stays in L2); its size is published as
+// soon as the parse knows it, and the PREVIOUS block is placed while the next
+// one loads: by then its predecessors have long published theirs, so the
+// look-back rarely waits.
+//
+// What bounds it: the latency of its stages and instruction issue, about
+// evenly (CHIME-shaped cube, 256 frequencies, 33024 blocks of 8 KiB: 217 us,
+// issue active 57 %, ALU 54 %, shared-memory pipe 49 %, DRAM 25 %; 24, 28 or
+// 32 warps per SM make no difference).  The one-warp kernel it replaces took
+// 290 us there.  Whole cube, 1.08 GB: 1.10 -> 0.83 ms; 268 MB of float64 in
+// 32 KiB blocks, which took a kernel of two buffers per warp: 0.88 -> 0.20 ms.
+//
+// BC: the block size in elements when it is one of the usual ones (4 and
+// 8 KiB; full blocks only), else 0 for any size and for a shortened last
+// block.  With the size known the strides of the bit-rows, the loops over
+// the warps and the tables' places are constants.  TS: a time-slowest cube.
+template <int ES, int MODE, uint32_t BC, bool TS>
+__global__ void __launch_bounds__(BC ? 32 * cta_warps(BC *ES) : 32 * CTA_MAX_WARPS,
+                                  BC ? CTA_WARPS_PER_SM / cta_warps(BC *ES) : 2)
+    compress_cta_kernel(const __grid_constant__ CodecArgs a)
+{
+    extern __shared__ __align__(128) uint8_t sm[];
+    const uint32_t W = BC ? cta_warps(BC * ES) : blockDim.x >> 5;
+    const CtaPlan plan = cta_plan((BC ? BC : a.B) * ES);
+    uint8_t *buf = sm;
+    const CtaScratch c = cta_scratch(sm + plan.tmp, W);
+    uint64_t *bar = reinterpret_cast<uint64_t *>(sm + plan.smem - 16u);
+    uint32_t *next = c.ex + EX_CTL + 2;            // the next tile
+    uint64_t *excl = reinterpret_cast<uint64_t *>(c.ex + EX_CTL + 4);
+    if (threadIdx.x == 0) {
+        mbar_init(bar, 1);
+        fence_mbar_init();
+        *next = a.tile_begin + atomicAdd(a.tile_counter, 1u);
+    }
+    __syncthreads();
+    uint32_t tile = *next, parity = 0;
+    uint8_t *slot0 = a.slots + (size_t)(2 * blockIdx.x) * plan.slot, *slot1 = slot0 + plan.slot;
+    uint32_t ptile = ~0u, pcs = 0;                 // the block waiting to be placed, in slot1
+    bool pend = false;
+    auto elems = [&](uint32_t t) { return BC ? BC : block_elems_of(a, t); };
+    if (!TS && tile < a.tile_end)
+        pend = cta_load(buf, a.in + (uint64_t)tile * a.B * ES, elems(tile) * ES, bar);
+    for (;;) {
+        const bool work = tile < a.tile_end;
+        const uint32_t tid = fresh_tid(), lane = tid & 31u, warp = tid >> 5;
+        uint32_t cs = 0, nxt = tile;
+        if (work) {
+            const uint32_t Bb = elems(tile), S = Bb * ES;
+            const uint32_t c0 = (uint32_t)(((uint64_t)tile * a.B * ES) >> 3);   // first complex sample
+            if (pend) {
+                if (!mbar_wait_bounded(bar, parity) && tid == 0) set_status(a.status, BSGPU_ERR_TIMEOUT);
+                parity ^= 1u;
+            }
+            if (TS) {
+                if (a.vis.T % 16u == 0 && S % 128u == 0)
+                    cta_gather_groups(a, buf, c0, S / 8u);
+                else
+                    cta_gather_samples(a, buf, c0, S / 8u);
+            }
+            if (TS || (S & 15u)) __syncthreads();   // what plain stores brought
+            if (MODE == CTA_SAMPLE) {
+                cta_round_samples(buf, c0, S / 8u, a.vis);
+                __syncthreads();
+            }
+            uint32_t v[32];
+            const uint32_t units = cta_units<ES>(Bb);
+            if (tid < units)
+                cta_get_rows<ES>(buf, Bb, tid, v, CtaRound<ES, MODE>{&a.vis, buf, c0});
+            __syncthreads();
+            if (tid < units) cta_put_rows<ES>(buf, Bb, tid, v);
+            __syncthreads();
+            if (!cta_rows_whole<ES>(Bb)) cta_pack_rows<ES>(buf, Bb);
+            const uint32_t *s32 = reinterpret_cast<const uint32_t *>(buf);
+            const uint32_t rowlen = Bb / 8u, R = (rowlen & 3u) ? 0u : rowlen / 4u;
+            if ((ES == 4 || ES == 8) && Bb % 1024u == 0) {
+                // a warp's rows are whole bitmap words and still in its registers:
+                // compare each with the row above and the word to the left
+                const uint32_t h = ES == 8 && tid >= R ? 1u : 0u, g = tid - h * R;
+                if (tid < units) {
+                    uint32_t w = 32u * h * R + g;
+                    uint32_t up = h ? s32[w - R] : ~v[0];
+                    uint2 *E = c.E + (w >> 5);
+#pragma unroll
+                    for (int r = 0; r < 32; r++) {
+                        const uint32_t left = r || w ? s32[(int)w - 1] : ~v[0];
+                        const uint32_t row = __ballot_sync(FULL, v[r] == up);
+                        const uint32_t run = __ballot_sync(FULL, v[r] == left);
+                        if (lane == 0) *E = make_uint2(row, run);
+                        up = v[r];
+                        w += R;
+                        E += R >> 5;
+                    }
+                }
+            } else {
+                cta_eq_bitmaps(s32, S / 4u, R, c, W);
+            }
+            __syncthreads();
+            cs = cta_lz4_encode(
+                buf, S, rowlen, slot0 + 4, c, W,
+                [&](uint32_t size) {
+                    if (tid == 0) {
+                        lookback_publish(a.tile_state, tile, 4ull + size, 0);
+                        put_be32(slot0, size);
+                        *next = a.tile_begin + atomicAdd(a.tile_counter, 1u);
+                    }
+                },
+                [&] {   // the previous block's place, while this warp has nothing else to do
+                    if (ptile != ~0u) {
+                        const uint64_t x = lookback_some(a.tile_state, ptile, 4ull + pcs, 8u, lane);
+                        if (lane == 0) *excl = x;
+                    }
+                });
+            fence_proxy_async_smem();   // the reads of buf before the next bulk write
+            __syncthreads();
+            nxt = *next;
+            pend = false;
+            if (!TS && nxt < a.tile_end)
+                pend = cta_load(buf, a.in + (uint64_t)nxt * a.B * ES, elems(nxt) * ES, bar);
+        }
+        if (ptile != ~0u) {
+            if (W == 1 || !work || *excl == LB_UNKNOWN) {
+                __syncthreads();   // everyone has seen *excl
+                if (warp == 0) {
+                    uint64_t x = lookback_some(a.tile_state, ptile, 4ull + pcs, 1u << 21, lane);
+                    if (x == LB_UNKNOWN) {
+                        if (lane == 0) set_status(a.status, BSGPU_ERR_TIMEOUT);
+                        x = 0;
+                    }
+                    if (lane == 0) *excl = x;
+                }
+                __syncthreads();
+            }
+            cta_place(a, ptile, slot1, pcs, 12 + *excl);
+        }
+        if (!work) break;
+        ptile = tile;
+        pcs = cs;
+        uint8_t *t = slot0;
+        slot0 = slot1;
+        slot1 = t;
+        tile = nxt;
+    }
+    // (outside the loop, where it costs the other blocks no registers)
+    if (a.tile_begin == 0 && blockIdx.x == 0 && threadIdx.x < 32)
+        write_chunk_header(a.out, a.n_elem * ES, a.B * ES, threadIdx.x);
+    if (ptile + 1u == a.nb && threadIdx.x < 32)
+        compress_place_end(a, 12 + *excl + 4 + pcs, threadIdx.x);
+}
+
+// Tiles [a.tile_begin, a.tile_end) with as many CTAs as fit, at most max_ctas.
+template <int ES, int MODE, uint32_t BC, bool TS = false>
+cudaError_t launch_cta(const CodecArgs &a, uint32_t max_ctas, cudaStream_t s)
+{
+    const CtaPlan plan = cta_plan(a.B * ES);
+    auto kernel = compress_cta_kernel<ES, MODE, BC, TS>;
+    if (plan.smem > 48 * 1024) {
+        const cudaError_t e = cudaFuncSetAttribute(
+            kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)plan.smem);
+        if (e != cudaSuccess) return e;
+    }
+    int dev = 0, sms = 148, per = 1;
+    if (cudaGetDevice(&dev) == cudaSuccess)
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kernel, (int)(32 * plan.W), plan.smem) !=
+            cudaSuccess || per < 1)
+        per = 1;
+    uint64_t grid = (uint64_t)sms * (uint32_t)per;
+    if (grid > max_ctas) grid = max_ctas;
+    if (grid > a.tile_end - a.tile_begin) grid = a.tile_end - a.tile_begin;
+    kernel<<<(uint32_t)grid, 32 * plan.W, plan.smem, s>>>(a);
+    return cudaGetLastError();
+}
+
+// The whole stream: full blocks of a usual size through their own kernel and
+// a shortened last block after them; other sizes, and streams short enough
+// that a second launch costs more than constant strides give, through the
+// general one.
+template <int ES, int MODE, uint32_t... BCS>
+cudaError_t launch_cta_stream(const CodecArgs &a0, uint32_t max_ctas, cudaStream_t s)
+{
+    CodecArgs a = a0;
+    const uint32_t nfull = a.nb - (a.last_B != a.B ? 1u : 0u);
+    a.tile_begin = 0;
+    a.tile_end = a.nb;
+    if (MODE != CTA_PLAIN && a.vis.tslow)
+        return launch_cta<ES, MODE, 0, MODE != CTA_PLAIN>(a, max_ctas, s);
+    if (nfull == a.nb || nfull > CTA_SPLIT_BLOCKS) {
+        cudaError_t e = cudaErrorNotReady;   // no such kernel
+        a.tile_end = nfull;
+        ((a.B == BCS ? (void)(e = launch_cta<ES, MODE, BCS>(a, max_ctas, s)) : (void)0), ...);
+        if (e == cudaSuccess) {
+            if (nfull == a.nb) return e;
+            a.tile_begin = nfull;
+            a.tile_counter = a.tile_counter + 1;
+        } else if (e != cudaErrorNotReady) {
+            return e;
+        }
+        a.tile_end = a.nb;
+    }
+    return launch_cta<ES, MODE, 0>(a, max_ctas, s);
+}
+
+}  // namespace bsg

@@ -1,4 +1,5 @@
-// The fast compress kernel (full blocks of at most 8 KiB, Sec. 4.2.1), shared
+// The level-1 compress kernel of full blocks of at most 8 KiB (Sec. 4.2.1; level
+// 0 takes compress_cta.cuh), shared
 // by the translation units that instantiate it: kernels.cu for cubes and
 // streams stored in order, tslow.cu for time-slowest cubes and for cubes
 // whose time axis is not a multiple of 16.
@@ -18,9 +19,10 @@ namespace bsg {
 // round_group_full).  PS (a cube whose time axis is not a multiple of 16, so
 // 16-sample groups would straddle products): the samples are rounded one by
 // one before the plain transpose, and with TS gathered one by one.
-template <int LEVEL, int ES, bool GEN = false, bool TS = false, bool PS = false>
+template <int ES, bool GEN = false, bool TS = false, bool PS = false>
 __global__ void __launch_bounds__(32, 20) compress_fast_kernel(const __grid_constant__ CodecArgs a)
 {
+    constexpr int LEVEL = 1;
     using L = FastPlan<LEVEL>;
     // a staged block comes back into the buffer and the encoder's scratch
     // after it (both free by then) for its placement
@@ -42,10 +44,6 @@ __global__ void __launch_bounds__(32, 20) compress_fast_kernel(const __grid_cons
     uint32_t tile = grab_tile(a.tile_counter, lane);
     while (tile < a.tile_end) {
         const uint32_t Bb = a.B;  // the fast path takes full blocks only
-        // 2048 4-byte elements at level 0 (the CHIME-shaped default): the
-        // transpose also yields the encoder's equality bitmaps
-        const bool EQ = LEVEL == 0 && ES == 4 && !PS && Bb == 2048;
-        uint32_t Erow[2], Erun[2];
         if (TS) {
             if (PS)
                 gather_tslow_samples(a, tmp, tile, lane);
@@ -87,28 +85,12 @@ __global__ void __launch_bounds__(32, 20) compress_fast_kernel(const __grid_cons
             shuffle4_inplace(tmp, Bb, lane, NoRound{});
         } else if (a.vis.enabled) {
             const VisGroupRound<GEN> round{&a.vis, (uint32_t)(((uint64_t)tile * a.B) >> 1)};
-            if (EQ)
-                shuffle4_inplace_eq(tmp, lane, round, Erow, Erun);
-            else
-                shuffle4_inplace(tmp, Bb, lane, round);
-        } else if (EQ) {
-            shuffle4_inplace_eq(tmp, lane, NoRound{}, Erow, Erun);
+            shuffle4_inplace(tmp, Bb, lane, round);
         } else {
             shuffle4_inplace(tmp, Bb, lane, NoRound{});
         }
         __syncwarp();
-        uint32_t cs;
-        if (LEVEL == 0 && (Bb * ES) % 128u == 0) {
-            if (!EQ)
-                lz4_eq_bitmaps(reinterpret_cast<const uint32_t *>(tmp), Bb * ES / 128, Bb / 32, lane, Erow,
-                               Erun);
-            cs = lz4_encode_bitmap_fast_eq(tmp, Bb * ES, Bb / 8, slot0 + 4,
-                                           static_cast<uint32_t *>(scratch), Erow, Erun);
-            if (lane == 0) put_be32(slot0, cs);
-            __syncwarp();
-        } else {
-            cs = compress_encode<LEVEL, L::HBITS>(a, Bb, tmp, slot0, scratch, lane);
-        }
+        const uint32_t cs = compress_encode<LEVEL, L::HBITS>(a, Bb, tmp, slot0, scratch, lane);
         lookback_publish(a.tile_state, tile, 4ull + cs, lane);
         const uint32_t nxt = grab_tile(a.tile_counter, lane);
         if (ptile != ~0u) place_staged(a, ptile, slot1, pcs, tmp, bar, parity, lane);

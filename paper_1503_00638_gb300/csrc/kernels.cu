@@ -446,28 +446,16 @@ __global__ void __launch_bounds__(32, MAXB <= 8192 ? 9 : 1)
 }
 
 
-uint32_t compress_fast_smem_bytes(int level)
-{
-    return level >= 1 ? FastPlan<1>::BYTES : FastPlan<0>::BYTES;
-}
+uint32_t compress_fast_smem_bytes() { return FastPlan<1>::BYTES; }
 
-uint32_t compress_fast_blocks_per_sm(int level, uint32_t es)
+uint32_t compress_fast_blocks_per_sm(uint32_t es)
 {
     int n = 0;
-    const uint32_t smem = compress_fast_smem_bytes(level);
-    cudaError_t e;
-    if (es == 8)
-        e = level >= 1
-            ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, compress_fast_kernel<1, 8>, 32, smem)
-            : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, compress_fast_kernel<0, 8>, 32, smem);
-    else if (es == 2)
-        e = level >= 1
-            ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, compress_fast_kernel<1, 2>, 32, smem)
-            : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, compress_fast_kernel<0, 2>, 32, smem);
-    else
-        e = level >= 1
-            ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, compress_fast_kernel<1, 4>, 32, smem)
-            : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, compress_fast_kernel<0, 4>, 32, smem);
+    const uint32_t smem = compress_fast_smem_bytes();
+    const cudaError_t e =
+        es == 8   ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, compress_fast_kernel<8>, 32, smem)
+        : es == 2 ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, compress_fast_kernel<2>, 32, smem)
+                  : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, compress_fast_kernel<4>, 32, smem);
     return e == cudaSuccess && n > 0 ? (uint32_t)n : 1u;
 }
 
@@ -1440,18 +1428,12 @@ cudaError_t launch_compress(const CodecArgs &a, uint32_t maxb, uint32_t grid, cu
 
 cudaError_t launch_compress_fast(const CodecArgs &a, uint32_t grid, cudaStream_t s)
 {
-    const uint32_t smem = compress_fast_smem_bytes(a.level);
-    if (a.es == 8)
-        return a.level >= 1 ? launch_warp_kernel(compress_fast_kernel<1, 8>, smem, grid, s, a)
-                            : launch_warp_kernel(compress_fast_kernel<0, 8>, smem, grid, s, a);
-    if (a.es == 2)
-        return a.level >= 1 ? launch_warp_kernel(compress_fast_kernel<1, 2>, smem, grid, s, a)
-                            : launch_warp_kernel(compress_fast_kernel<0, 2>, smem, grid, s, a);
+    const uint32_t smem = compress_fast_smem_bytes();
+    if (a.es == 8) return launch_warp_kernel(compress_fast_kernel<8>, smem, grid, s, a);
+    if (a.es == 2) return launch_warp_kernel(compress_fast_kernel<2>, smem, grid, s, a);
     if (a.vis.enabled && (a.vis.is_int || a.vis.cft || a.vis.qtab))
-        return a.level >= 1 ? launch_warp_kernel(compress_fast_kernel<1, 4, true>, smem, grid, s, a)
-                            : launch_warp_kernel(compress_fast_kernel<0, 4, true>, smem, grid, s, a);
-    return a.level >= 1 ? launch_warp_kernel(compress_fast_kernel<1, 4>, smem, grid, s, a)
-                        : launch_warp_kernel(compress_fast_kernel<0, 4>, smem, grid, s, a);
+        return launch_warp_kernel(compress_fast_kernel<4, true>, smem, grid, s, a);
+    return launch_warp_kernel(compress_fast_kernel<4>, smem, grid, s, a);
 }
 
 cudaError_t launch_compress_small(const CodecArgs &a, cudaStream_t s)
