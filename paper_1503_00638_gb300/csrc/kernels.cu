@@ -5,6 +5,8 @@
 // bulk-copy (TMA) engine with the next block prefetched.
 #include <cuda_runtime.h>
 
+#include <cstring>
+
 #include "compress_fast.cuh"
 
 namespace bsg {
@@ -201,11 +203,37 @@ __global__ void __launch_bounds__(256) vis_compensation_kernel(const void *__res
 // fp64 instruction works (on GB300 fp64 issues at a small fraction of the
 // fp32 rate, and a warp instruction costs the same whatever its lanes).
 // Per sample: V's lower triangle; Cholesky V = L L^H in place (of -V when
-// V_00 < 0); X = L^-1 in place, column by column (for column j, every L
-// entry still needed lies right of it or below the current row); W = X^H X
-// for the diagonal and for each product.  The q table is [F][M][T], so the
-// lanes' writes (consecutive times) coalesce.
-__device__ __forceinline__ uint32_t tri_el(uint32_t r, uint32_t c) { return r * (r + 1) / 2 + c; }
+// V_00 < 0), of whose diagonal only the reciprocals are needed; X = L^-1 in
+// place, column by column (for column j, every L entry still needed lies
+// right of it or below the current row); W = X^H X for the diagonal and for
+// each product.  The q table is [F][M][T], so the lanes' writes (consecutive
+// times) coalesce.
+//
+// Bound by the fp64 pipe, so what does not need 64 bits stays out of it: the
+// products are chains of fused multiply-adds (four a complex product, no
+// separate subtraction), 1 / L_jj is one reciprocal square root, and q is
+// taken from W in float32 wherever its granularity is beyond doubt.  8
+// inputs, 1024 x 64 samples: 217 us, 366 us with a fp64 division per component
+// (64 per sample) and separate additions.
+BSG_HD uint32_t tri_el(uint32_t r, uint32_t c) { return r * (r + 1) / 2 + c; }
+
+// q = fl32(12 f / h) where h = N2 (ww + re2), N2 = N or 2 N, ww = W_ii W_jj
+// and re2 = +-Re(W_ij^2).  The rounding only asks for the k of 4^k < q: a
+// float32 quotient answers that unless a power of four lies within 256 units
+// in the last place (at least 2^-16 of q; the quotient's error is below 100
+// units of 2^-24: some 18 roundings relative to ww, which h exceeds by 0.2 at
+// least), or the sum cancels, or something leaves the middle of the float
+// range; then the quotient is taken in fp64.
+BSG_HD bool q_beyond_doubt(float q, float ww, float h)
+{
+#ifdef __CUDA_ARCH__
+    const uint32_t Q = __float_as_uint(q);
+#else
+    uint32_t Q;
+    memcpy(&Q, &q, 4);
+#endif
+    return h > 0.2f * ww && q > 1e-30f && q < 1e30f && magic_bits(Q - 256u) == magic_bits(Q + 256u);
+}
 
 __global__ void __launch_bounds__(32) full_noise_kernel(const void *__restrict__ vis, VisParams P,
                                                         uint32_t n_freq, double f, double N,
@@ -216,6 +244,7 @@ __global__ void __launch_bounds__(32) full_noise_kernel(const void *__restrict__
     const uint32_t n = P.n_in, NP = P.P, M = P.M;   // NP = n (n + 1) / 2 triangle elements
     double *Ar = fsm + lane, *Ai = fsm + 32 * NP + lane, *D = fsm + 64 * NP + lane;
     float *qtab = const_cast<float *>(P.qtab);
+    const float f12 = (float)(12.0 * f / N);
     const uint64_t n_smp = (uint64_t)n_freq * P.T;
     for (uint64_t base = (uint64_t)blockIdx.x * 32; base < n_smp; base += (uint64_t)gridDim.x * 32) {
         const uint64_t smp = base + lane;
@@ -223,72 +252,84 @@ __global__ void __launch_bounds__(32) full_noise_kernel(const void *__restrict__
         const uint32_t fr = live ? (uint32_t)(smp / P.T) : 0u, t = live ? (uint32_t)(smp % P.T) : 0u;
         bool ok = live;
         if (live) {
+#pragma unroll 4
             for (uint32_t p = 0; p < NP; p++) {
                 const uint32_t ij = __ldg(P.pairs + p), i = ij & 0xffffu, j = ij >> 16;
-                const size_t at = vis_src(P, ((size_t)fr * NP + p) * P.T + t) * 2;
+                const size_t at = vis_src(P, ((size_t)fr * NP + p) * P.T + t);
+                const uint2 v = __ldg(reinterpret_cast<const uint2 *>(vis) + at);
                 double re, im;   // the stored values (int32 through float32)
                 if (P.is_int) {
-                    re = (double)(float)__ldg(reinterpret_cast<const int32_t *>(vis) + at);
-                    im = (double)(float)__ldg(reinterpret_cast<const int32_t *>(vis) + at + 1);
+                    re = (double)(float)(int32_t)v.x;
+                    im = (double)(float)(int32_t)v.y;
                 } else {
-                    re = __ldg(reinterpret_cast<const float *>(vis) + at);
-                    im = __ldg(reinterpret_cast<const float *>(vis) + at + 1);
+                    re = __uint_as_float(v.x);
+                    im = __uint_as_float(v.y);
                 }
                 Ar[32 * tri_el(j, i)] = re;   // V_ji = conj(V_ij)
                 Ai[32 * tri_el(j, i)] = -im;
             }
             const double sg = Ar[0] < 0.0 ? -1.0 : 1.0;
             for (uint32_t j = 0; j < n; j++) {
-                double d = sg * Ar[32 * tri_el(j, j)];
+                const double *Ljr = Ar + 32 * tri_el(j, 0), *Lji = Ai + 32 * tri_el(j, 0);
+                double d = sg * Ljr[32 * j];
                 for (uint32_t k = 0; k < j; k++) {
-                    const double lr = Ar[32 * tri_el(j, k)], li = Ai[32 * tri_el(j, k)];
-                    d -= lr * lr + li * li;
+                    const double lr = Ljr[32 * k], li = Lji[32 * k];
+                    d = fma(-lr, lr, d);
+                    d = fma(-li, li, d);
                 }
                 if (!(d > 0.0) || !isfinite(d)) {
                     ok = false;
                     break;
                 }
-                const double ljj = sqrt(d), rl = 1.0 / ljj;
-                Ar[32 * tri_el(j, j)] = ljj;
-                Ai[32 * tri_el(j, j)] = 0.0;
+                const double rl = rsqrt(d);
                 D[32 * j] = rl;
                 for (uint32_t i = j + 1; i < n; i++) {
                     // (sg V_ij - sum_{k<j} L_ik conj(L_jk)) / L_jj
-                    double sr = sg * Ar[32 * tri_el(i, j)], si = sg * Ai[32 * tri_el(i, j)];
+                    double *Lir = Ar + 32 * tri_el(i, 0), *Lii = Ai + 32 * tri_el(i, 0);
+                    double sr = sg * Lir[32 * j], si = sg * Lii[32 * j];
                     for (uint32_t k = 0; k < j; k++) {
-                        const double ar = Ar[32 * tri_el(i, k)], ai = Ai[32 * tri_el(i, k)];
-                        const double br = Ar[32 * tri_el(j, k)], bi = Ai[32 * tri_el(j, k)];
-                        sr -= ar * br + ai * bi;
-                        si -= ai * br - ar * bi;
+                        const double ar = Lir[32 * k], ai = Lii[32 * k];
+                        const double br = Ljr[32 * k], bi = Lji[32 * k];
+                        sr = fma(-ar, br, sr);
+                        si = fma(-ai, br, si);
+                        sr = fma(-ai, bi, sr);
+                        si = fma(ar, bi, si);
                     }
-                    Ar[32 * tri_el(i, j)] = sr * rl;
-                    Ai[32 * tri_el(i, j)] = si * rl;
+                    Lir[32 * j] = sr * rl;
+                    Lii[32 * j] = si * rl;
                 }
             }
         }
         if (ok) {
             // X_jj = 1 / L_jj, X_ij = -(sum_{j<=k<i} L_ik X_kj) / L_ii
             for (uint32_t j = 0; j < n; j++) {
-                Ar[32 * tri_el(j, j)] = D[32 * j];
+                const double xjj = D[32 * j];
                 for (uint32_t i = j + 1; i < n; i++) {
-                    double ur = 0.0, ui = 0.0;
-                    for (uint32_t k = j; k < i; k++) {
-                        const double ar = Ar[32 * tri_el(i, k)], ai = Ai[32 * tri_el(i, k)];
+                    double *Lir = Ar + 32 * tri_el(i, 0), *Lii = Ai + 32 * tri_el(i, 0);
+                    double ur = Lir[32 * j] * xjj, ui = Lii[32 * j] * xjj;
+                    for (uint32_t k = j + 1; k < i; k++) {
+                        const double ar = Lir[32 * k], ai = Lii[32 * k];
                         const double xr = Ar[32 * tri_el(k, j)], xi = Ai[32 * tri_el(k, j)];
-                        ur += ar * xr - ai * xi;
-                        ui += ar * xi + ai * xr;
+                        ur = fma(ar, xr, ur);
+                        ui = fma(ar, xi, ui);
+                        ur = fma(-ai, xi, ur);
+                        ui = fma(ai, xr, ui);
                     }
-                    const double rli = D[32 * i];
-                    Ar[32 * tri_el(i, j)] = -ur * rli;
-                    Ai[32 * tri_el(i, j)] = -ui * rli;
+                    const double rli = -D[32 * i];
+                    Lir[32 * j] = ur * rli;
+                    Lii[32 * j] = ui * rli;
                 }
+                Ar[32 * tri_el(j, j)] = xjj;
+                Ai[32 * tri_el(j, j)] = 0.0;
             }
             // W_ii = sum_{k >= i} |X_ki|^2 (D is free again)
             for (uint32_t i = 0; i < n; i++) {
-                double w = 0.0;
-                for (uint32_t k = i; k < n; k++) {
+                const double x = Ar[32 * tri_el(i, i)];
+                double w = x * x;
+                for (uint32_t k = i + 1; k < n; k++) {
                     const double xr = Ar[32 * tri_el(k, i)], xi = Ai[32 * tri_el(k, i)];
-                    w += xr * xr + xi * xi;
+                    w = fma(xr, xr, w);
+                    w = fma(xi, xi, w);
                 }
                 D[32 * i] = w;
             }
@@ -296,30 +337,41 @@ __global__ void __launch_bounds__(32) full_noise_kernel(const void *__restrict__
         if (live) {
             for (uint32_t p = 0; p < NP; p++) {
                 const uint32_t ij = __ldg(P.pairs + p), i = ij & 0xffffu, j = ij >> 16;
-                double hre = 0.0, him = 0.0;   // (C^-1)_kk of the Re and Im components
-                if (ok) {
-                    const double wi = D[32 * i];
-                    if (i == j) {
-                        hre = N * (wi * wi);
-                    } else {
-                        double wr = 0.0, wm = 0.0;   // W_ij = sum_{k >= j} conj(X_ki) X_kj
-                        for (uint32_t k = j; k < n; k++) {
-                            const double ar = Ar[32 * tri_el(k, i)], ai = Ai[32 * tri_el(k, i)];
-                            const double br = Ar[32 * tri_el(k, j)], bi = Ai[32 * tri_el(k, j)];
-                            wr += ar * br + ai * bi;
-                            wm += ar * bi - ai * br;
-                        }
-                        const double ww = wi * D[32 * j], re2 = wr * wr - wm * wm;
-                        hre = 2.0 * N * (ww + re2);
-                        him = 2.0 * N * (ww - re2);
+                double wr = 0.0, wm = 0.0;   // W_ij = sum_{k >= j} conj(X_ki) X_kj
+                if (ok && i != j) {
+                    const double x = Ar[32 * tri_el(j, j)];
+                    wr = Ar[32 * tri_el(j, i)] * x;
+                    wm = -(Ai[32 * tri_el(j, i)] * x);
+                    for (uint32_t k = j + 1; k < n; k++) {
+                        const double ar = Ar[32 * tri_el(k, i)], ai = Ai[32 * tri_el(k, i)];
+                        const double br = Ar[32 * tri_el(k, j)], bi = Ai[32 * tri_el(k, j)];
+                        wr = fma(ar, br, wr);
+                        wm = fma(ar, bi, wm);
+                        wr = fma(ai, bi, wr);
+                        wm = fma(-ai, br, wm);
                     }
                 }
+                const double wi = ok ? D[32 * i] : 0.0, wj = ok ? D[32 * j] : 0.0;
+                const float wif = (float)wi, wjf = (float)wj, wrf = (float)wr, wmf = (float)wm;
+                const float wwf = wif * wjf, re2f = (wrf - wmf) * (wrf + wmf);
                 for (int part = 0; part < 2; part++) {
                     if (part == 1 && i == j) break;
                     const uint32_t comp = part ? NP + p - i - 1 : p;
-                    const double s2 = ok ? 1.0 / (part ? him : hre) : 0.0;
-                    qtab[((size_t)fr * M + comp) * P.T + t] = ok ? (float)(12.0 * f * s2) : 0.0f;
-                    if (s2_out) s2_out[smp * M + comp] = s2;
+                    float q = 0.0f;
+                    if (ok) {
+                        const float hf = i == j ? wwf : 2.0f * (part ? wwf - re2f : wwf + re2f);
+                        q = __fdividef(f12, hf);
+                        if (s2_out || !(fminf(wif, wjf) > 1e-30f) || !q_beyond_doubt(q, wwf, hf)) {
+                            const double ww = wi * wj, re2 = wr * wr - wm * wm;
+                            const double h = i == j ? N * ww : 2.0 * N * (part ? ww - re2 : ww + re2);
+                            const double s2 = 1.0 / h;   // 1 / (C^-1)_kk
+                            q = (float)(12.0 * f * s2);
+                            if (s2_out) s2_out[smp * M + comp] = s2;
+                        }
+                    } else if (s2_out) {
+                        s2_out[smp * M + comp] = 0.0;
+                    }
+                    qtab[((size_t)fr * M + comp) * P.T + t] = q;
                 }
             }
         }
