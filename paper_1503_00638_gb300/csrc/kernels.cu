@@ -66,6 +66,10 @@ __global__ void vis_tables_kernel(const float *__restrict__ vis, VisParams V, ui
         // int32 autos are converted to float32 (round to nearest)
         autos[x] = is_int ? __int2float_rn(reinterpret_cast<const int32_t *>(vis)[at]) : vis[at];
     }
+    if (V.cft)   // the quotients of vis_compensation_kernel start at 0
+        for (uint64_t x = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; x < (uint64_t)n_freq * T;
+             x += stride)
+            const_cast<float *>(V.cft)[x] = 0.0f;
     for (uint64_t p = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; p < P; p += stride) {
         // row i holds products [i n - i (i-1)/2, (i+1) n - (i+1) i / 2)
         uint32_t lo = 0, hi = n_in - 1;
@@ -83,42 +87,93 @@ __global__ void vis_tables_kernel(const float *__restrict__ vis, VisParams V, ui
 // Sec. 3.2's compensation: per (freq, time) sample, c is recomputed from
 // f m with m = min over cross products of 1 - |V_ij|^2 / (V_ii V_jj) in
 // float32 (each operation rounded to nearest; a negative or NaN value counts
-// as 0; no cross product gives 1), c = fl32(6 (f m) / N) in fp64.  One CTA per
-// (frequency, chunk of up to 1024 time samples); the minimum of non-negative
-// floats is taken on their bit patterns (order-free, so per-thread minima
-// merged by one atomic each give the same result as any other order).
-__global__ void __launch_bounds__(256) vis_compensation_kernel(const void *__restrict__ vis,
-                                                               VisParams P, float *cft,
-                                                               uint32_t n_freq, double f,
-                                                               double N)
+// as 0; no cross product gives 1), c = fl32(6 (f m) / N) in fp64.
+//
+// m follows from the largest rounded quotient, so a thread keeps that one and
+// divides only where a product may exceed it (a multiplication tells; the
+// margin covers its rounding): a division takes more instructions than all
+// the rest of a sample.  The threads of one time share what they have found
+// (a warp divides when any of its lanes does).  A CTA takes a slice of the
+// products of one frequency and up to 1024 times.  With one slice it writes c;
+// with more (few frequencies would leave SMs idle: 128 CTAs for 128
+// frequencies took 104 us, 135 MB at 1.3 TB/s; 42 us now) the quotients meet in the
+// table by atomics on the bits of non-negative floats, order-free, and
+// vis_compensation_end_kernel turns them into c.
+struct CompMax {
+    float q;   // the largest quotient so far (0 at first); +inf once one was NaN
+    BSG_D void add(float re, float im, float Ai, float Aj)
+    {
+        const float num = __fadd_rn(__fmul_rn(re, re), __fmul_rn(im, im));
+        const float den = __fmul_rn(Ai, Aj);
+        if (den > 1e-30f && num < __fmul_rn(__fmul_rn(q, den), 0.999999f)) return;
+        const float r = __fdiv_rn(num, den);
+        q = r == r ? fmaxf(q, r) : __int_as_float(0x7f800000);
+    }
+    // exchange with the other threads of the same time
+    BSG_D void share(volatile uint32_t *best)
+    {
+        const uint32_t other = *best, own = __float_as_uint(q);
+        if (own > other)
+            atomicMax(const_cast<uint32_t *>(best), own);
+        else
+            q = __uint_as_float(other);
+    }
+};
+
+// c from the largest quotient's bits
+BSG_D float compensated_c(uint32_t q_bits, double f, double N)
 {
-    __shared__ uint32_t mins[1024];
+    const float om = __fsub_rn(1.0f, __uint_as_float(q_bits));
+    const double fe = __dmul_rn(f, (double)(om >= 0.0f ? om : 0.0f));
+    return __double2float_rn(__ddiv_rn(__dmul_rn(6.0, fe), N));
+}
+
+template <bool INT>
+BSG_D float2 comp_sample(uint2 v)
+{
+    return INT ? make_float2(__int2float_rn((int32_t)v.x), __int2float_rn((int32_t)v.y))
+               : make_float2(__uint_as_float(v.x), __uint_as_float(v.y));
+}
+
+template <bool INT>
+__global__ void __launch_bounds__(256) vis_compensation_kernel(const uint2 *__restrict__ vis,
+                                                               VisParams P, float *cft,
+                                                               uint32_t n_freq, uint32_t slices,
+                                                               double f, double N)
+{
+    __shared__ uint32_t best[1024];   // bits of the largest quotient per time
     const uint32_t nchunk = (P.T + 1023) / 1024;
-    for (uint32_t cb = blockIdx.x; cb < n_freq * nchunk; cb += gridDim.x) {
+    const uint32_t sl = blockIdx.x % slices, per_slice = (P.P + slices - 1) / slices;
+    const uint32_t p_lo = sl * per_slice, p_hi = p_lo + per_slice < P.P ? p_lo + per_slice : P.P;
+    for (uint32_t cb = blockIdx.x / slices; cb < n_freq * nchunk; cb += gridDim.x / slices) {
         const uint32_t fr = cb / nchunk, t0 = (cb % nchunk) * 1024;
         const uint32_t tn = P.T - t0 < 1024 ? P.T - t0 : 1024;
-        for (uint32_t t = threadIdx.x; t < tn; t += blockDim.x) mins[t] = __float_as_uint(1.0f);
+        uint32_t *table = reinterpret_cast<uint32_t *>(cft + (size_t)fr * P.T + t0);
+        // (with several slices, what the others have found so far)
+        for (uint32_t t = threadIdx.x; t < tn; t += blockDim.x)
+            best[t] = slices == 1 ? 0u : *(volatile uint32_t *)(table + t);
         __syncthreads();
-        if (!P.tslow && tn <= blockDim.x) {
-            // time-fastest cube: thread (p0, tl) takes time t0 + tl of products
-            // p0, p0 + per, ... (the lanes of a product read consecutive
-            // samples), keeps its minimum in a register and merges it once
-            const uint32_t per = blockDim.x / tn, tl = threadIdx.x % tn, p0 = threadIdx.x / tn;
-            if (p0 < per) {
+        if (!P.tslow) {
+            // time-fastest cube: thread (p0, tl) takes time t0 + tl (and tl +
+            // 256, ... of a long axis) of products p0, p0 + per, ...; the
+            // lanes of a product read consecutive samples.  Eight samples (and
+            // their product entries) are loaded before any is used, with no
+            // branch between the loads, so that they are in flight together.
+            const uint32_t tw = tn < blockDim.x ? tn : blockDim.x;
+            const uint32_t per = blockDim.x / tw, p0 = threadIdx.x / tw;
+            for (uint32_t tl = threadIdx.x % tw; tl < tn && p0 < per; tl += tw) {
                 const uint32_t t = t0 + tl;
                 const float *arow = P.autos + (size_t)fr * P.n_in * P.T + t;
-                uint32_t m = __float_as_uint(1.0f);
-                // eight samples (and their product entries) are loaded before
-                // any is used, with no branch between the loads, so that they
-                // are in flight together
-                const uint2 *vrow = reinterpret_cast<const uint2 *>(vis) + (size_t)fr * P.P * P.T + t;
-                for (uint32_t pb = p0; pb < P.P; pb += 8 * per) {
+                const uint2 *vrow = vis + (size_t)fr * P.P * P.T + t;
+                CompMax m{0.0f};
+                for (uint32_t pb = p_lo + p0; pb < p_hi; pb += 8 * per) {
+                    m.share(best + tl);
                     uint2 v[8];
                     uint32_t ijs[8];
 #pragma unroll
                     for (uint32_t k = 0; k < 8; k++) {
                         const uint32_t p = pb + k * per;
-                        const bool in = p < P.P;
+                        const bool in = p < p_hi;
                         v[k] = in ? __ldg(vrow + (size_t)p * P.T) : make_uint2(0u, 0u);
                         ijs[k] = in ? __ldg(P.pairs + p) : 0u;   // 0: the auto (0, 0), skipped
                     }
@@ -126,55 +181,60 @@ __global__ void __launch_bounds__(256) vis_compensation_kernel(const void *__res
                     for (uint32_t k = 0; k < 8; k++) {
                         const uint32_t i = ijs[k] & 0xffffu, j = ijs[k] >> 16;
                         if (i == j) continue;
-                        const float Ai = __ldg(arow + (size_t)i * P.T);
-                        const float Aj = __ldg(arow + (size_t)j * P.T);
-                        float re, im;
-                        if (P.is_int) {
-                            re = __int2float_rn((int32_t)v[k].x);
-                            im = __int2float_rn((int32_t)v[k].y);
-                        } else {
-                            re = __uint_as_float(v[k].x);
-                            im = __uint_as_float(v[k].y);
-                        }
-                        const float num = __fadd_rn(__fmul_rn(re, re), __fmul_rn(im, im));
-                        const float den = __fmul_rn(Ai, Aj);
-                        float om = __fsub_rn(1.0f, __fdiv_rn(num, den));
-                        if (!(om >= 0.0f)) om = 0.0f;
-                        m = min(m, __float_as_uint(om));
+                        const float2 x = comp_sample<INT>(v[k]);
+                        m.add(x.x, x.y, __ldg(arow + (size_t)i * P.T), __ldg(arow + (size_t)j * P.T));
                     }
                 }
-                atomicMin(&mins[tl], m);
+                m.share(best + tl);
             }
-        } else
-        for (uint64_t e = threadIdx.x; e < (uint64_t)P.P * tn; e += blockDim.x) {
-            const uint32_t p = (uint32_t)(e / tn), t = t0 + (uint32_t)(e % tn);
-            const uint32_t ij = __ldg(P.pairs + p);
-            const uint32_t i = ij & 0xffffu, j = ij >> 16;
-            if (i == j) continue;
-            const float Ai = __ldg(P.autos + ((size_t)fr * P.n_in + i) * P.T + t);
-            const float Aj = __ldg(P.autos + ((size_t)fr * P.n_in + j) * P.T + t);
-            const size_t at = vis_src(P, ((size_t)fr * P.P + p) * P.T + t) * 2;
-            float re, im;
-            if (P.is_int) {
-                re = __int2float_rn(reinterpret_cast<const int32_t *>(vis)[at]);
-                im = __int2float_rn(reinterpret_cast<const int32_t *>(vis)[at + 1]);
-            } else {
-                re = reinterpret_cast<const float *>(vis)[at];
-                im = reinterpret_cast<const float *>(vis)[at + 1];
+        } else {
+            // time-slowest cube: a warp takes one time and its lanes
+            // consecutive products, which are neighbours in the input
+            for (uint32_t tl = threadIdx.x >> 5; tl < tn; tl += blockDim.x >> 5) {
+                const uint32_t t = t0 + tl;
+                const float *arow = P.autos + (size_t)fr * P.n_in * P.T + t;
+                const uint2 *vrow = vis + (size_t)t * P.FP + (size_t)fr * P.P;
+                CompMax m{0.0f};
+                for (uint32_t pb = p_lo + (threadIdx.x & 31u); pb < p_hi; pb += 4 * 32) {
+                    m.q = __uint_as_float(__reduce_max_sync(__activemask(), __float_as_uint(m.q)));
+                    uint2 v[4];
+                    uint32_t ijs[4];
+#pragma unroll
+                    for (uint32_t k = 0; k < 4; k++) {
+                        const uint32_t p = pb + 32 * k;
+                        const bool in = p < p_hi;
+                        v[k] = in ? __ldg(vrow + p) : make_uint2(0u, 0u);
+                        ijs[k] = in ? __ldg(P.pairs + p) : 0u;
+                    }
+#pragma unroll
+                    for (uint32_t k = 0; k < 4; k++) {
+                        const uint32_t i = ijs[k] & 0xffffu, j = ijs[k] >> 16;
+                        if (i == j) continue;
+                        const float2 x = comp_sample<INT>(v[k]);
+                        m.add(x.x, x.y, __ldg(arow + (size_t)i * P.T), __ldg(arow + (size_t)j * P.T));
+                    }
+                }
+                m.share(best + tl);
             }
-            const float num = __fadd_rn(__fmul_rn(re, re), __fmul_rn(im, im));
-            const float den = __fmul_rn(Ai, Aj);
-            float om = __fsub_rn(1.0f, __fdiv_rn(num, den));
-            if (!(om >= 0.0f)) om = 0.0f;
-            atomicMin(&mins[t - t0], __float_as_uint(om));
         }
         __syncthreads();
         for (uint32_t t = threadIdx.x; t < tn; t += blockDim.x) {
-            const double fe = __dmul_rn(f, (double)__uint_as_float(mins[t]));
-            cft[(size_t)fr * P.T + t0 + t] = __double2float_rn(__ddiv_rn(__dmul_rn(6.0, fe), N));
+            if (slices == 1)
+                cft[(size_t)fr * P.T + t0 + t] = compensated_c(best[t], f, N);
+            else
+                atomicMax(table + t, best[t]);
         }
         __syncthreads();
     }
+}
+
+// The table of quotients to c, after the slices have met.
+__global__ void __launch_bounds__(256) vis_compensation_end_kernel(float *cft, uint64_t n, double f,
+                                                                   double N)
+{
+    for (uint64_t k = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; k < n;
+         k += (uint64_t)gridDim.x * blockDim.x)
+        cft[k] = compensated_c(__float_as_uint(cft[k]), f, N);
 }
 
 // Sec. 3.1's full covariance for small arrays (Eq. rad_full1-3) and the noise
@@ -1310,10 +1370,32 @@ __global__ void __launch_bounds__(32) shuffle_kernel(const __grid_constant__ Cod
 cudaError_t launch_vis_compensation(const void *vis, const VisParams &P, uint32_t n_freq,
                                     double f, double N, cudaStream_t s)
 {
+    int dev = 0, sms = 148;
+    if (cudaGetDevice(&dev) == cudaSuccess)
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     const uint64_t work = (uint64_t)n_freq * ((P.T + 1023) / 1024);
-    const uint32_t grid = (uint32_t)(work < 8192 ? work : 8192);
-    vis_compensation_kernel<<<grid ? grid : 1, 256, 0, s>>>(vis, P, const_cast<float *>(P.cft),
-                                                            n_freq, f, N);
+    // slices of the products: enough CTAs for the eight that are resident per
+    // SM, each thread still with eight samples or more (twice or four times
+    // as many CTAs: 3 and 10 % slower, each starting from less knowledge of
+    // the maximum)
+    const uint64_t want = ((uint64_t)sms * 8 + work - 1) / work;
+    uint64_t most = (uint64_t)P.P * (P.T < 256 ? P.T : 256) / (256 * 8);
+    if (most < 1) most = 1;
+    const uint32_t slices = (uint32_t)(want < most ? want : most);
+    float *cft = const_cast<float *>(P.cft);
+    const uint64_t n = (uint64_t)n_freq * P.T;
+    const uint64_t cap = 65536 / slices;
+    const uint32_t grid = (uint32_t)((work < cap ? work : cap) * slices);
+    if (P.is_int)
+        vis_compensation_kernel<true><<<grid, 256, 0, s>>>(reinterpret_cast<const uint2 *>(vis), P,
+                                                           cft, n_freq, slices, f, N);
+    else
+        vis_compensation_kernel<false><<<grid, 256, 0, s>>>(reinterpret_cast<const uint2 *>(vis), P,
+                                                            cft, n_freq, slices, f, N);
+    if (slices > 1) {
+        const uint64_t b = (n + 255) / 256;
+        vis_compensation_end_kernel<<<(uint32_t)(b < 4096 ? b : 4096), 256, 0, s>>>(cft, n, f, N);
+    }
     return cudaGetLastError();
 }
 

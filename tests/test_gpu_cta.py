@@ -83,3 +83,20 @@ def test_cube_streams_equal_rounding_then_compressing(shape, dtype, tslow):
             torch.cuda.synchronize()
             assert c.nbytes == int(nb.item())
             assert torch.equal(c.buf[:c.nbytes], out[:c.nbytes])
+
+
+@pytest.mark.parametrize("shape", [(1, 40, 300), (2, 128, 1), (3, 24, 1100), (1, 90, 33)])
+def test_compensated_f_over_slices_of_the_products(orc, shape):
+    """The minimum over the products taken slice by slice, in both orders and
+    over time axes longer than a CTA, bit for bit the oracle's."""
+    from paper_1503_00638_gb300 import bsgpu, synth
+    F, n, T = shape
+    cfg = synth.VisConfig(F, n, T, 2 ** 14, 0.05, seed=n, rho=0.6)
+    v = synth.visibilities(cfg)
+    v[0, 5] = np.complex64(complex(np.nan, 1.0)) if T > 1000 else v[0, 5]
+    want = orc.reduce_precision(v, cfg.n_samp, cfg.f, True).view(np.uint32)
+    d = torch.from_numpy(v).cuda()
+    for tslow in (False, True):
+        x = d.permute(2, 0, 1).contiguous() if tslow else d
+        got = bsgpu.reduce_precision(x, cfg.n_samp, cfg.f, True, time_slowest=tslow)
+        assert np.array_equal(got.cpu().numpy().view(np.uint32), want)
