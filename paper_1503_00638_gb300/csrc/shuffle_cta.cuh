@@ -77,40 +77,7 @@ BSG_D void cta_get_rows(const uint8_t *buf, uint32_t Bb, uint32_t u, uint32_t (&
     } else if (ES == 2) {
         shuf2_read_group(buf + 128u * u, u & 7u, v);
     } else {
-        // Word n of the transpose's input takes elements n, n + 32, n + 64 and
-        // n + 96 (a 4 x 4 byte transpose of words i, i + 8, i + 16, i + 24),
-        // so that word 8 s + r of its output is bits 32 s .. 32 s + 31 of
-        // bit-row r.  The 16-byte chunk 2 b + p (b: which 32 elements, p:
-        // which half) is read with p flipped by f and b rotated by t from lane
-        // to lane, which spreads the lanes over the banks here and in
-        // cta_put_rows; f comes out as a rotation of the words by 16 bits,
-        // undone here, t as the order of the four words, undone there.
-        const uint32_t f = (u >> 2) & 1u, t = ((u & 3u) + (u >> 3)) & 3u;
-        const uint4 *s4 = reinterpret_cast<const uint4 *>(buf + 128u * u);
-#pragma unroll
-        for (uint32_t p = 0; p < 2; p++) {
-            uint32_t w[4][4];
-#pragma unroll
-            for (uint32_t b = 0; b < 4; b++) {
-                const uint4 q = s4[2u * ((b + t) & 3u) + (p ^ f)];
-                w[b][0] = q.x;
-                w[b][1] = q.y;
-                w[b][2] = q.z;
-                w[b][3] = q.w;
-            }
-#pragma unroll
-            for (uint32_t i = 0; i < 4; i++) {
-                const uint32_t a = bperm(w[0][i], w[1][i], 0x5140), b = bperm(w[0][i], w[1][i], 0x7362);
-                const uint32_t d = bperm(w[2][i], w[3][i], 0x5140), e = bperm(w[2][i], w[3][i], 0x7362);
-                v[16 * p + 4 * i] = bperm(a, d, 0x5410);
-                v[16 * p + 4 * i + 1] = bperm(a, d, 0x7632);
-                v[16 * p + 4 * i + 2] = bperm(b, e, 0x5410);
-                v[16 * p + 4 * i + 3] = bperm(b, e, 0x7632);
-            }
-        }
-        transpose32(v);
-#pragma unroll
-        for (int r = 0; r < 32; r++) v[r] = rotl(v[r], 16u * f);
+        shuf1_read_group(buf + 128u * u, u, v);
     }
 }
 
@@ -128,13 +95,7 @@ BSG_D void cta_put_rows(uint8_t *buf, uint32_t Bb, uint32_t u, const uint32_t (&
     } else if (ES == 2) {
         shuf2_put_rows(buf, (Bb + 63u) / 64u, u, v, 0, 16);
     } else {
-        const uint32_t t = ((u & 3u) + (u >> 3)) & 3u, row = 4u * ((Bb + 127u) / 128u);
-#pragma unroll
-        for (uint32_t s = 0; s < 4; s++) {
-            uint32_t *p = d32 + 4u * u + ((s + t) & 3u);
-#pragma unroll
-            for (uint32_t r = 0; r < 8; r++, p += row) *p = v[8 * s + r];
-        }
+        shuf1_put_rows(buf, 4u * ((Bb + 127u) / 128u), u, v);
     }
 }
 
