@@ -800,22 +800,17 @@ __global__ void __launch_bounds__(32, 20) decompress_inplace_kernel(const __grid
     __syncwarp();
 }
 
-// In-place decoding for the shapes the 8 KiB kernel does not take (blocks
-// over 8 KiB, 1-byte elements): one buffer per warp with the block's
-// compressed image near its end and the bit-rows decoded from its start,
-// un-transposed from there straight into the output, which is 16-byte
-// aligned for every block (the caller checks B * es).  The margin argument
-// above holds for any S: the LZ4 bytes must start at least 2 + 2 S / 255
-// bytes after S - clen, and dec_issue puts them at least E - clen - 47
-// bytes in (E the buffer size), so E >= S + 2 S / 255 + 49 suffices
-// (inplace_any_buf gives S + 2 S / 255 + 160).  Half the shared memory of
-// decompress_kernel, which holds the compressed and the decoded block apart:
-// twice the resident warps or more.
-template <uint32_t MAXB>
-__global__ void __launch_bounds__(32, MAXB <= 8192 ? 20 : (MAXB <= 16384 ? 12 : (MAXB <= 32768 ? 6 : 3)))
-    decompress_inplace_any_kernel(const __grid_constant__ CodecArgs a)
+// In-place decoding for 1-byte elements in blocks of at most 8 KiB: one buffer
+// per warp with the block's compressed image near its end and the bit-rows
+// decoded from its start, un-transposed from there straight into the output,
+// which is 16-byte aligned for every block (the caller checks B * es).  The
+// margin argument above holds for any S: the LZ4 bytes must start at least 2 +
+// 2 S / 255 bytes after S - clen, and dec_issue puts them at least E - clen -
+// 47 bytes in (E the buffer size), so E >= S + 2 S / 255 + 49 suffices.
+// (Blocks over 8 KiB: decompress_cta.cuh.)
+__global__ void __launch_bounds__(32, 20) decompress_inplace_any_kernel(const __grid_constant__ CodecArgs a)
 {
-    constexpr uint32_t BUF = inplace_any_buf(MAXB);
+    constexpr uint32_t BUF = INPLACE_BUF;
     extern __shared__ __align__(128) uint8_t sm[];
     uint8_t *buf = sm;
     uint64_t *bar = reinterpret_cast<uint64_t *>(sm + BUF);
@@ -876,10 +871,7 @@ __global__ void __launch_bounds__(32, MAXB <= 8192 ? 20 : (MAXB <= 16384 ? 12 : 
     }
 }
 
-uint32_t decompress_inplace_any_smem_bytes(uint32_t maxb)
-{
-    return inplace_any_buf(maxb) + 16;
-}
+uint32_t decompress_inplace_any_smem_bytes() { return INPLACE_BUF + 16; }
 
 uint32_t decompress_inplace_blocks_per_sm(uint32_t es)
 {
@@ -1647,14 +1639,9 @@ cudaError_t launch_decompress(const CodecArgs &a, uint32_t maxb, uint32_t grid, 
     return launch_warp_kernel(decompress_kernel<65536, 0>, smem, grid, s, a);
 }
 
-cudaError_t launch_decompress_inplace_any(const CodecArgs &a, uint32_t maxb, uint32_t grid,
-                                          cudaStream_t s)
+cudaError_t launch_decompress_inplace_any(const CodecArgs &a, uint32_t grid, cudaStream_t s)
 {
-    const uint32_t smem = decompress_inplace_any_smem_bytes(maxb);
-    if (maxb <= 8192) return launch_warp_kernel(decompress_inplace_any_kernel<8192>, smem, grid, s, a);
-    if (maxb <= 16384) return launch_warp_kernel(decompress_inplace_any_kernel<16384>, smem, grid, s, a);
-    if (maxb <= 32768) return launch_warp_kernel(decompress_inplace_any_kernel<32768>, smem, grid, s, a);
-    return launch_warp_kernel(decompress_inplace_any_kernel<65536>, smem, grid, s, a);
+    return launch_warp_kernel(decompress_inplace_any_kernel, decompress_inplace_any_smem_bytes(), grid, s, a);
 }
 
 cudaError_t launch_chain_walk(const CodecArgs &a, uint64_t *offsets, void *seg_ws,

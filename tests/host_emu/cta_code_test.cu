@@ -1,13 +1,16 @@
 // CPU test of the CTA-wide device code of paper_1503_00638_gb300/csrc (the
-// in-place bit transpose and the level-0 LZ4 encoder) on the CTA emulator:
-// the transpose against the oracle's, the encoder byte for byte against the
-// one-warp encoder's parse (lz4_encode_bitmap, run on a CTA of one warp) and
-// through the oracle's decoder.  argv: element size, elements, kind, seed.
+// in-place bit transpose, the level-0 LZ4 encoder and the two-warp decoder)
+// on the CTA emulator: the transpose against the oracle's, the encoder byte
+// for byte against the one-warp encoder's parse (lz4_encode_bitmap, run on a
+// CTA of one warp) and through the oracle's decoder, the decoder in place on
+// both encoders' blocks and, for its verdict, on damaged ones.  argv: element size, elements, kind, seed.
 #include "cta_emu.h"
 #include "../../paper_1503_00638_gb300/csrc/lz4_cta.cuh"
+#include "../../paper_1503_00638_gb300/csrc/lz4_cta_dec.cuh"
 #include "../../paper_1503_00638_gb300/csrc/shuffle_cta.cuh"
 #include <random>
 extern "C" {
+size_t orc_lz4_compress_block(const uint8_t *src, size_t n, uint8_t *dst, size_t cap);
 int orc_lz4_decompress_block(const uint8_t *src, size_t src_len, uint8_t *dst, size_t dst_len);
 int orc_bitshuffle(const void *vin, void *vout, size_t n, size_t es, size_t block_elems, int inverse);
 }
@@ -23,6 +26,24 @@ template <int ES> static void transpose(uint32_t Bb)
     if (u < units) cta_put_rows<ES>(buf, Bb, u, v);
     __syncthreads();
     if (!cta_rows_whole<ES>(Bb)) cta_pack_rows<ES>(buf, Bb);
+}
+
+// The block's image at phase `ph` near the end of the buffer, as the kernel
+// places it, decoded to the buffer's start by two warps.
+static bool decode_in_place(const uint8_t *img, uint32_t cs, uint32_t S, uint32_t ph)
+{
+    alignas(16) static uint8_t D[70000];
+    alignas(16) static uint32_t ring[DEC_RING_WORDS];
+    const uint32_t E = (S + 2u * S / 255u + 160u + 15u) & ~15u, off = (E - (cs + 4u) - 32u) & ~15u;
+    memset(D, 0x5A, sizeof D);
+    memcpy(D + off + ph + 4, img, cs);
+    bool ok = false;
+    run_cta(64, [&] {
+        const bool r = cta_lz4_decode(D, off + ph + 4, cs, D, S, ring, threadIdx.x);
+        if (threadIdx.x == 0) ok = r;
+    });
+    memcpy(buf, D, S);
+    return ok;
 }
 
 int main(int argc, char **argv)
@@ -92,6 +113,29 @@ int main(int argc, char **argv)
     if (orc_lz4_decompress_block(enc, cs, back.data(), S) || memcmp(back.data(), rows.data(), S)) {
         fprintf(stderr, "the oracle rejects the block\n");
         return 1;
+    }
+    std::vector<uint8_t> oc(lz4_bound(S) + 16);
+    const uint32_t ocs = (uint32_t)orc_lz4_compress_block(rows.data(), S, oc.data(), oc.size());
+    for (int who = kind & 1; who < 2; who++)   // (the CTA's threads are real ones: slow)
+        for (uint32_t ph : {who ? 5u : 15u})
+            if (!decode_in_place(who ? oc.data() : enc, who ? ocs : cs, S, ph) || memcmp(buf, rows.data(), S)) {
+                fprintf(stderr, "decoding in place differs, phase %u, encoder %d\n", ph, who);
+                return 1;
+            }
+    // a byte changed, the end cut off: the verdict of the oracle's decoder
+    for (int t = 0; t < (S <= 4096 && kind < 2 ? 3 : 0); t++) {
+        std::vector<uint8_t> bad(oc.begin(), oc.begin() + ocs);
+        if (t % 3 == 2)
+            bad.resize(rng() % bad.size());
+        else
+            bad[rng() % bad.size()] = (uint8_t)rng();
+        const bool want_ok = !bad.empty() && orc_lz4_decompress_block(bad.data(), bad.size(), back.data(), S) == 0;
+        std::vector<uint8_t> img(bad);
+        img.resize(bad.size() + 16, 0xEE);
+        if (decode_in_place(img.data(), (uint32_t)bad.size(), S, 3) != want_ok) {
+            fprintf(stderr, "verdict on a damaged block differs (%d)\n", t);
+            return 1;
+        }
     }
     printf("ok %u -> %u\n", S, cs);
     return 0;
