@@ -241,7 +241,7 @@ def run_reference(args, rank):
 
 # the sources the profiled compress kernel is compiled from
 KERNEL_SOURCES = ("kernels.cu", "kernels.cuh", "compress_cta.cuh", "lz4_cta.cuh",
-                  "shuffle_cta.cuh", "compress_fast.cuh", "codec.cuh", "common.cuh",
+                  "shuffle_cta.cuh", "codec.cuh", "common.cuh",
                   "lz4_warp.cuh", "shuffle.cuh")
 
 

@@ -19,7 +19,7 @@ LIBDIR = os.path.join(HERE, "lib")
 LIB = os.path.join(LIBDIR, "libbsgpu.so")
 INCLUDE = os.path.join(os.path.dirname(HERE), "include")
 SOURCES = ["kernels.cu", "compress_cta.cu", "compress_cta12.cu", "compress_cta8.cu",
-           "compress_cta_vis.cu", "decompress_cta.cu", "compress_cta_visx.cu", "tslow.cu", "batch.cu", "capi.cu", "noalloc.cu", "arena.cpp"]
+           "compress_cta_vis.cu", "decompress_cta.cu", "compress_cta_visx.cu", "compress_cta_l1.cu", "compress_cta_l1_vis.cu", "batch.cu", "capi.cu", "noalloc.cu", "arena.cpp"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 NVCC_FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC,-O2",
               "-Xptxas", "-O3"]

@@ -181,7 +181,7 @@ template <int LEVEL>
 __host__ __device__ constexpr uint32_t batch_compress_warp_smem() { return r128(FastPlan<LEVEL>::BYTES); }
 __host__ __device__ constexpr uint32_t batch_decompress_warp_smem() { return r128(INPLACE_BUF + 16); }
 
-// Persistent, one shared buffer per warp (as compress_fast_kernel): per
+// Persistent, one shared buffer per warp (bulk copy, transpose in place, LZ4): per
 // item, transpose the block, LZ4-encode it into this warp's staging slot,
 // publish its size in its chunk's look-back state, then place the PREVIOUS
 // item's block, whose predecessors have long published theirs.  Only the

@@ -88,13 +88,12 @@ uint32_t persistent_grid(uint32_t smem_per_cta, uint64_t work)
 }
 
 struct WsLayout {
-    size_t state, autos, pairs, cft, qtab, offsets, segs, slots, gslots, total;
-    uint32_t gslot_warps;  // warps the general compressor's slots cover
-    size_t cslots;         // staging slots of the level-0 compressor (the same space)
-    uint32_t cslot_ctas;   // CTAs they cover
+    size_t state, autos, pairs, cft, qtab, offsets, segs, gslots, cslots, total;
+    uint32_t gslot_warps;  // warps the general compressor's slots (gslots) cover
+    uint32_t cslot_ctas;   // CTAs the compressor's slots (cslots) cover
 };
 
-// SMs the general compressor's staging slots are sized for (at least the
+// SMs the compressors' staging slots are sized for (at least the
 // device's count; GB300 has 152)
 constexpr uint32_t GEN_MAX_SMS = 160;
 
@@ -118,13 +117,6 @@ VisOpts vis_opts(int flags, int64_t n_freq, int64_t n_in, int64_t n_time)
     return o;
 }
 
-// Whether level-1 compress takes the fast kernel: full blocks of at most 8 KiB
-// of 2-, 4- or 8-byte elements (a cube in any order, any time axis).
-bool fast_shape(const Geometry &g)
-{
-    return shuffle_inplace_ok(g.es, g.B);
-}
-
 // n_ft: entries of the per-(freq, time) compensated-c table (0 = none)
 WsLayout ws_layout(int op, const Geometry &g, size_t n_auto, size_t n_prod, uint64_t n_time = 0,
                    const VisOpts &opts = VisOpts())
@@ -134,35 +126,25 @@ WsLayout ws_layout(int op, const Geometry &g, size_t n_auto, size_t n_prod, uint
     if (op == BSGPU_OP_COMPRESS || op == BSGPU_OP_COMPRESS_VIS) {
         L.state = o;
         o += r256((size_t)g.nb * 8);
-        const size_t slots0 = o;
-        if (g.nb && fast_shape(g)) {
-            L.slots = o;
-            o += (size_t)FAST_MAX_WARPS * 2 * FAST_SLOT_BYTES;
-        }
-        // the general compressor's staging slots: for its one shortened last
-        // block after the fast path, else for as many warps as can be
-        // resident (at most GEN_MAX_SMS SMs)
-        const uint32_t gwork = !g.nb ? 0u : fast_shape(g) ? (g.last_B != g.B ? 1u : 0u) : g.nb;
-        if (gwork) {
+        if (g.nb && compress_cta_ok(g.es, g.B)) {
+            // two staging slots for every CTA that can be resident (at most
+            // GEN_MAX_SMS SMs)
+            uint64_t ctas = compress_cta_max(g.B * g.es, GEN_MAX_SMS);
+            if (ctas > g.nb) ctas = g.nb;
+            L.cslots = o;
+            L.cslot_ctas = (uint32_t)ctas;
+            o += r256(compress_cta_slots_bytes(g.B * g.es, L.cslot_ctas));
+        } else if (g.nb) {
+            // the general compressor's, for as many warps
             const uint32_t maxb = maxb_class(g.B * g.es);
             const uint32_t smem = compress_smem_bytes(maxb, 0, true);
             uint32_t per_sm = (228u * 1024u) / (smem + 1024u);
             if (per_sm == 0) per_sm = 1;
             uint64_t w = (uint64_t)GEN_MAX_SMS * per_sm;
-            if (w > gwork) w = gwork;
+            if (w > g.nb) w = g.nb;
             L.gslots = o;
             L.gslot_warps = (uint32_t)w;
             o += r256((size_t)w * 2 * compress_slot_bytes(maxb));
-        }
-        // the level-0 compressor's slots take the place of the other two's
-        // (a call uses one or the other)
-        if (g.nb && compress_cta_ok(g.es, g.B)) {
-            uint64_t ctas = compress_cta_max(g.B * g.es, GEN_MAX_SMS);
-            if (ctas > g.nb) ctas = g.nb;
-            L.cslots = slots0;
-            L.cslot_ctas = (uint32_t)ctas;
-            const size_t end = slots0 + r256(compress_cta_slots_bytes(g.B * g.es, L.cslot_ctas));
-            if (o < end) o = end;
         }
     }
     if (op == BSGPU_OP_COMPRESS_VIS || op == BSGPU_OP_REDUCE_PRECISION) {
@@ -464,47 +446,17 @@ static int compress_common(const void *in, const Geometry &g, int level, void *o
     if (cudaMemsetAsync(ws, 0, L.state + (size_t)g.nb * 8, s) != cudaSuccess)
         return BSGPU_ERR_CUDA;
     if (g.nb == 0) return cuda_err(launch_compress_small(a, s));
-    if (level == 0 && L.cslots) {
+    if (L.cslots) {
         a.slots = reinterpret_cast<uint8_t *>(ws) + L.cslots;
         return cuda_err(launch_compress_cta(a, L.cslot_ctas, s));
     }
-    // level 1: full blocks through the fast kernel when its slots are in the
-    // workspace, the rest (a shortened last block, other shapes) through the
-    // general one; both place blocks through the same look-back state
-    const uint32_t nfull = g.nb - (g.last_B != g.B ? 1u : 0u);
-    uint32_t done = 0;
-    if (L.slots && nfull) {
-        int dev = 0, sms = 148;
-        if (cudaGetDevice(&dev) == cudaSuccess)
-            cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        const bool ts = vis && vis->tslow;
-        // 4-byte components of a cube whose time axis is not a multiple of 16
-        const bool ps = vis && !vis->tslow && g.es == 4 && (vis->T % 16u) != 0;
-        uint64_t grid = (uint64_t)sms * (ts ? compress_fast_tslow_blocks_per_sm(g.es)
-                                            : ps ? compress_fast_ps_blocks_per_sm()
-                                                 : compress_fast_blocks_per_sm(g.es));
-        if (grid > nfull) grid = nfull;
-        if (grid > FAST_MAX_WARPS) grid = FAST_MAX_WARPS;
-        CodecArgs f = a;
-        f.tile_begin = 0;
-        f.tile_end = nfull;
-        f.slots = reinterpret_cast<uint8_t *>(ws) + L.slots;
-        f.nslot_warps = FAST_MAX_WARPS;
-        f.tile_counter = reinterpret_cast<uint32_t *>((uint8_t *)ws + 4);
-        cudaError_t e = ts   ? launch_compress_fast_tslow(f, (uint32_t)grid, s)
-                        : ps ? launch_compress_fast_ps(f, (uint32_t)grid, s)
-                             : launch_compress_fast(f, (uint32_t)grid, s);
-        if (e != cudaSuccess) return BSGPU_ERR_CUDA;
-        done = nfull;
-    }
-    if (done == g.nb) return BSGPU_OK;
-    a.tile_begin = done;
+    // block sizes whose bit-rows are no whole words: the general kernel
+    a.tile_begin = 0;
     a.tile_end = g.nb;
-    a.tile_counter = reinterpret_cast<uint32_t *>((uint8_t *)ws + 8);
     uint32_t maxb = maxb_class(g.B * g.es);
     a.slots = L.gslots ? reinterpret_cast<uint8_t *>(ws) + L.gslots : nullptr;
     a.nslot_warps = L.gslot_warps;
-    uint32_t grid = persistent_grid(compress_smem_bytes(maxb, level, a.slots != nullptr), g.nb - done);
+    uint32_t grid = persistent_grid(compress_smem_bytes(maxb, level, a.slots != nullptr), g.nb);
     if (a.slots && grid > a.nslot_warps) grid = a.nslot_warps;
     return cuda_err(launch_compress(a, maxb, grid, s));
 }

@@ -1,4 +1,4 @@
-// The level-0 compress kernel: [gather ->] round -> bit-transpose -> LZ4 ->
+// The compress kernel: [gather ->] round -> bit-transpose -> LZ4 ->
 // placement of one block per CTA step (Sec. 4.2.1, Sec. 6 steps 1-5), for
 // every element size, every block size up to 64 KiB whose bit-rows are whole
 // words (cta_shape_ok), and the shortened last block of such a stream.
@@ -32,10 +32,25 @@ struct CtaPlan {
     uint32_t smem;       // dynamic shared memory
     uint32_t slot;       // bytes of a staging slot
 };
+// Warps of level 1: two units of 128 bytes to a thread.  Its search is one
+// warp's work and shared memory, with the hash table in it, holds 16 blocks of
+// 8 KiB per SM whatever the warps, so a second warp per block only took
+// registers, and what counts is that the search keeps its values in them: 67
+// MB of 16-bit walks in 8 KiB blocks take 245 us at 128 registers a thread,
+// 305 at 112, 317 at 96, 326 at 80 (the one-warp kernel that wrote each
+// sequence before it searched on: 299), 364 us with two warps at 64.
+template <int LEVEL>
+__host__ __device__ constexpr uint32_t cta_warps_of(uint32_t S)
+{
+    return LEVEL >= 1 ? (S + 8191u) / 8192u : cta_warps(S);
+}
+
+template <int LEVEL>
 __host__ __device__ constexpr CtaPlan cta_plan(uint32_t S)
 {
-    const uint32_t W = cta_warps(S), tmp = r16(S + 16u);
-    return CtaPlan{W, tmp, tmp + r16(cta_scratch_bytes(W)) + 16u, r16(4u + lz4b(S) + 32u)};
+    const uint32_t W = cta_warps_of<LEVEL>(S), tmp = r16(S + 16u);
+    return CtaPlan{W, tmp, tmp + r16(cta_scratch_bytes<LEVEL>(W, cta_hbits(S))) + 16u,
+                   r16(4u + lz4b(S) + 32u)};
 }
 
 // Round 16 complex samples in registers (v[m] = component (m + 4 rot) mod 32
@@ -171,8 +186,9 @@ BSG_D void cta_gather_samples(const CodecArgs &a, uint8_t *buf, uint32_t c0, uin
 
 // A time axis that is a multiple of 16: thread q takes 16-sample series
 // groups q, q + NT, ... (neighbouring threads, neighbouring series), their
-// 16-byte chunks in an order rotated by lane / 4 for whole sectors and
-// distinct banks (as gather_tslow_block).
+// 16-byte chunks in an order rotated by lane / 4: at every step the four lanes
+// of one 32-byte sector of neighbouring series read the same time row, and the
+// chunks the 32 lanes store fall in eight different bank groups.
 BSG_D void cta_gather_groups(const CodecArgs &a, uint8_t *buf, uint32_t c0, uint32_t n)
 {
     const VisParams &P = a.vis;
@@ -318,16 +334,15 @@ BSG_D uint64_t lookback_some(uint64_t *state, uint32_t tile, uint64_t agg, uint3
 // 8 KiB; full blocks only), else 0 for any size and for a shortened last
 // block.  With the size known the strides of the bit-rows, the loops over
 // the warps and the tables' places are constants.  TS: a time-slowest cube.
-template <int ES, int MODE, uint32_t BC, bool TS>
-__global__ void __launch_bounds__(BC ? 32 * cta_warps(BC *ES) : 32 * CTA_MAX_WARPS,
-                                  BC ? CTA_WARPS_PER_SM / cta_warps(BC *ES) : 2)
-    compress_cta_kernel(const __grid_constant__ CodecArgs a)
+template <int LEVEL, int ES, int MODE, uint32_t BC, bool TS>
+BSG_D void compress_cta_body(const CodecArgs &a)
 {
     extern __shared__ __align__(128) uint8_t sm[];
     const uint32_t W = BC ? cta_warps(BC * ES) : blockDim.x >> 5;
-    const CtaPlan plan = cta_plan((BC ? BC : a.B) * ES);
+    const CtaPlan plan = cta_plan<LEVEL>((BC ? BC : a.B) * ES);
+    const uint32_t hbits = cta_hbits((BC ? BC : a.B) * ES);
     uint8_t *buf = sm;
-    const CtaScratch c = cta_scratch(sm + plan.tmp, W);
+    const CtaScratch c = cta_scratch<LEVEL>(sm + plan.tmp, W, hbits);
     uint64_t *bar = reinterpret_cast<uint64_t *>(sm + plan.smem - 16u);
     uint32_t *next = c.ex + EX_CTL + 2;            // the next tile
     uint64_t *excl = reinterpret_cast<uint64_t *>(c.ex + EX_CTL + 4);
@@ -366,31 +381,38 @@ __global__ void __launch_bounds__(BC ? 32 * cta_warps(BC *ES) : 32 * CTA_MAX_WAR
                 cta_round_samples(buf, c0, S / 8u, a.vis);
                 __syncthreads();
             }
-            uint32_t v[32];
+            constexpr uint32_t UPT = LEVEL >= 1 ? 2 : 1;   // units per thread
+            uint32_t v[UPT][32];
             const uint32_t units = cta_units<ES>(Bb);
-            if (tid < units)
-                cta_get_rows<ES>(buf, Bb, tid, v, CtaRound<ES, MODE>{&a.vis, buf, c0});
+#pragma unroll
+            for (uint32_t k = 0; k < UPT; k++)
+                if (tid + 32u * W * k < units)
+                    cta_get_rows<ES>(buf, Bb, tid + 32u * W * k, v[k], CtaRound<ES, MODE>{&a.vis, buf, c0});
             __syncthreads();
-            if (tid < units) cta_put_rows<ES>(buf, Bb, tid, v);
+#pragma unroll
+            for (uint32_t k = 0; k < UPT; k++)
+                if (tid + 32u * W * k < units) cta_put_rows<ES>(buf, Bb, tid + 32u * W * k, v[k]);
             __syncthreads();
             if (!cta_rows_whole<ES>(Bb)) cta_pack_rows<ES>(buf, Bb);
             const uint32_t *s32 = reinterpret_cast<const uint32_t *>(buf);
             const uint32_t rowlen = Bb / 8u, R = (rowlen & 3u) ? 0u : rowlen / 4u;
-            if ((ES == 4 || ES == 8) && Bb % 1024u == 0) {
+            if (LEVEL >= 1) {
+                // (no bitmaps)
+            } else if ((ES == 4 || ES == 8) && Bb % 1024u == 0) {
                 // a warp's rows are whole bitmap words and still in its registers:
                 // compare each with the row above and the word to the left
                 const uint32_t h = ES == 8 && tid >= R ? 1u : 0u, g = tid - h * R;
                 if (tid < units) {
                     uint32_t w = 32u * h * R + g;
-                    uint32_t up = h ? s32[w - R] : ~v[0];
+                    uint32_t up = h ? s32[w - R] : ~v[0][0];
                     uint2 *E = c.E + (w >> 5);
 #pragma unroll
                     for (int r = 0; r < 32; r++) {
-                        const uint32_t left = r || w ? s32[(int)w - 1] : ~v[0];
-                        const uint32_t row = __ballot_sync(FULL, v[r] == up);
-                        const uint32_t run = __ballot_sync(FULL, v[r] == left);
+                        const uint32_t left = r || w ? s32[(int)w - 1] : ~v[0][0];
+                        const uint32_t row = __ballot_sync(FULL, v[0][r] == up);
+                        const uint32_t run = __ballot_sync(FULL, v[0][r] == left);
                         if (lane == 0) *E = make_uint2(row, run);
-                        up = v[r];
+                        up = v[0][r];
                         w += R;
                         E += R >> 5;
                     }
@@ -398,9 +420,9 @@ __global__ void __launch_bounds__(BC ? 32 * cta_warps(BC *ES) : 32 * CTA_MAX_WAR
             } else {
                 cta_eq_bitmaps(s32, S / 4u, R, c, W);
             }
-            __syncthreads();
-            cs = cta_lz4_encode(
-                buf, S, rowlen, slot0 + 4, c, W,
+            if (LEVEL == 0) __syncthreads();
+            cs = cta_lz4_encode<LEVEL>(
+                buf, S, rowlen, slot0 + 4, c, W, hbits,
                 [&](uint32_t size) {
                     if (tid == 0) {
                         lookback_publish(a.tile_state, tile, 4ull + size, 0);
@@ -451,12 +473,32 @@ __global__ void __launch_bounds__(BC ? 32 * cta_warps(BC *ES) : 32 * CTA_MAX_WAR
         compress_place_end(a, 12 + *excl + 4 + pcs, threadIdx.x);
 }
 
+template <int ES, int MODE, uint32_t BC, bool TS>
+__global__ void __launch_bounds__(BC ? 32 * cta_warps(BC *ES) : 32 * CTA_MAX_WARPS,
+                                  BC ? CTA_WARPS_PER_SM / cta_warps(BC *ES) : 2)
+    compress_cta_kernel(const __grid_constant__ CodecArgs a)
+{
+    compress_cta_body<0, ES, MODE, BC, TS>(a);
+}
+
+// Level 1: shared memory bounds its CTAs, so a thread may have more registers
+// (see cta_warps_of).
+constexpr int CTA_L1_REGS = 128;
+
+template <int ES, int MODE, bool TS>
+__global__ void __maxnreg__(CTA_L1_REGS)
+    compress_cta_l1_kernel(const __grid_constant__ CodecArgs a)
+{
+    compress_cta_body<1, ES, MODE, 0, TS>(a);
+}
+
 // Tiles [a.tile_begin, a.tile_end) with as many CTAs as fit, at most max_ctas.
-template <int ES, int MODE, uint32_t BC, bool TS = false>
+template <int LEVEL, int ES, int MODE, uint32_t BC, bool TS = false>
 cudaError_t launch_cta(const CodecArgs &a, uint32_t max_ctas, cudaStream_t s)
 {
-    const CtaPlan plan = cta_plan(a.B * ES);
+    const CtaPlan plan = cta_plan<LEVEL>(a.B * ES);
     auto kernel = compress_cta_kernel<ES, MODE, BC, TS>;
+    if constexpr (LEVEL >= 1) kernel = compress_cta_l1_kernel<ES, MODE, TS>;
     if (plan.smem > 48 * 1024) {
         const cudaError_t e = cudaFuncSetAttribute(
             kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)plan.smem);
@@ -479,7 +521,7 @@ cudaError_t launch_cta(const CodecArgs &a, uint32_t max_ctas, cudaStream_t s)
 // a shortened last block after them; other sizes, and streams short enough
 // that a second launch costs more than constant strides give, through the
 // general one.
-template <int ES, int MODE, uint32_t... BCS>
+template <int LEVEL, int ES, int MODE, uint32_t... BCS>
 cudaError_t launch_cta_stream(const CodecArgs &a0, uint32_t max_ctas, cudaStream_t s)
 {
     CodecArgs a = a0;
@@ -487,11 +529,11 @@ cudaError_t launch_cta_stream(const CodecArgs &a0, uint32_t max_ctas, cudaStream
     a.tile_begin = 0;
     a.tile_end = a.nb;
     if (MODE != CTA_PLAIN && a.vis.tslow)
-        return launch_cta<ES, MODE, 0, MODE != CTA_PLAIN>(a, max_ctas, s);
-    if (nfull == a.nb || nfull > CTA_SPLIT_BLOCKS) {
+        return launch_cta<LEVEL, ES, MODE, 0, MODE != CTA_PLAIN>(a, max_ctas, s);
+    if (sizeof...(BCS) != 0 && (nfull == a.nb || nfull > CTA_SPLIT_BLOCKS)) {
         cudaError_t e = cudaErrorNotReady;   // no such kernel
         a.tile_end = nfull;
-        ((a.B == BCS ? (void)(e = launch_cta<ES, MODE, BCS>(a, max_ctas, s)) : (void)0), ...);
+        ((a.B == BCS ? (void)(e = launch_cta<LEVEL, ES, MODE, BCS>(a, max_ctas, s)) : (void)0), ...);
         if (e == cudaSuccess) {
             if (nfull == a.nb) return e;
             a.tile_begin = nfull;
@@ -501,7 +543,7 @@ cudaError_t launch_cta_stream(const CodecArgs &a0, uint32_t max_ctas, cudaStream
         }
         a.tile_end = a.nb;
     }
-    return launch_cta<ES, MODE, 0>(a, max_ctas, s);
+    return launch_cta<LEVEL, ES, MODE, 0>(a, max_ctas, s);
 }
 
 }  // namespace bsg

@@ -8,12 +8,12 @@ namespace bsg {
 
 cudaError_t launch_compress_cta_group_x(const CodecArgs &a, uint32_t max_ctas, cudaStream_t s)
 {
-    return launch_cta_stream<4, CTA_GROUP_X, 2048, 1024>(a, max_ctas, s);
+    return launch_cta_stream<0, 4, CTA_GROUP_X, 2048, 1024>(a, max_ctas, s);
 }
 
 cudaError_t launch_compress_cta_sample(const CodecArgs &a, uint32_t max_ctas, cudaStream_t s)
 {
-    return launch_cta_stream<4, CTA_SAMPLE, 2048, 1024>(a, max_ctas, s);
+    return launch_cta_stream<0, 4, CTA_SAMPLE, 2048, 1024>(a, max_ctas, s);
 }
 
 }  // namespace bsg

@@ -7,7 +7,7 @@
 
 #include <cstring>
 
-#include "compress_fast.cuh"
+#include "codec.cuh"
 
 namespace bsg {
 
@@ -555,20 +555,6 @@ __global__ void __launch_bounds__(32, MAXB <= 8192 ? 9 : 1)
         tile = nxt;
     }
     if (STAGED && ptile != ~0u) place_staged(a, ptile, slot1, pcs, tmp, bar2, parity2, lane);
-}
-
-
-uint32_t compress_fast_smem_bytes() { return FastPlan<1>::BYTES; }
-
-uint32_t compress_fast_blocks_per_sm(uint32_t es)
-{
-    int n = 0;
-    const uint32_t smem = compress_fast_smem_bytes();
-    const cudaError_t e =
-        es == 8   ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, compress_fast_kernel<8>, 32, smem)
-        : es == 2 ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, compress_fast_kernel<2>, 32, smem)
-                  : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, compress_fast_kernel<4>, 32, smem);
-    return e == cudaSuccess && n > 0 ? (uint32_t)n : 1u;
 }
 
 
@@ -1597,16 +1583,6 @@ cudaError_t launch_compress_t(const CodecArgs &a, uint32_t maxb, uint32_t grid, 
 cudaError_t launch_compress(const CodecArgs &a, uint32_t maxb, uint32_t grid, cudaStream_t s)
 {
     return a.slots ? launch_compress_t<true>(a, maxb, grid, s) : launch_compress_t<false>(a, maxb, grid, s);
-}
-
-cudaError_t launch_compress_fast(const CodecArgs &a, uint32_t grid, cudaStream_t s)
-{
-    const uint32_t smem = compress_fast_smem_bytes();
-    if (a.es == 8) return launch_warp_kernel(compress_fast_kernel<8>, smem, grid, s, a);
-    if (a.es == 2) return launch_warp_kernel(compress_fast_kernel<2>, smem, grid, s, a);
-    if (a.vis.enabled && (a.vis.is_int || a.vis.cft || a.vis.qtab))
-        return launch_warp_kernel(compress_fast_kernel<4, true>, smem, grid, s, a);
-    return launch_warp_kernel(compress_fast_kernel<4>, smem, grid, s, a);
 }
 
 cudaError_t launch_compress_small(const CodecArgs &a, cudaStream_t s)

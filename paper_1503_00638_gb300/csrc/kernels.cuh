@@ -108,22 +108,10 @@ cudaError_t launch_shuffle(const CodecArgs &a, bool inverse, uint32_t maxb, uint
 // a.nslot_warps) blocks are placed one block late from the slots; without,
 // each block is placed as soon as it is encoded.
 cudaError_t launch_compress(const CodecArgs &a, uint32_t maxb, uint32_t grid, cudaStream_t s);
-// Level 1, full blocks that the in-place register transposes take
-// (shuffle_inplace_ok; for a cube also n_time % 16 == 0): tiles
-// [0, a.tile_end), placement one block late through per-warp staging slots.
-cudaError_t launch_compress_fast(const CodecArgs &a, uint32_t grid, cudaStream_t s);
-uint32_t compress_fast_smem_bytes();
-uint32_t compress_fast_blocks_per_sm(uint32_t es);
-// the same for a time-slowest cube (n_time % 16 == 0), in tslow.cu
-cudaError_t launch_compress_fast_tslow(const CodecArgs &a, uint32_t grid, cudaStream_t s);
-uint32_t compress_fast_tslow_blocks_per_sm(uint32_t es);
-// the same for a time-fastest cube of 4-byte components with n_time % 16 != 0
-cudaError_t launch_compress_fast_ps(const CodecArgs &a, uint32_t grid, cudaStream_t s);
-uint32_t compress_fast_ps_blocks_per_sm();
-// staging slot size of the fast path and the warp count its slots cover
+// staging slot size of the batch compressor and the warp count its slots cover
 constexpr uint32_t FAST_SLOT_BYTES = 8304;
 constexpr uint32_t FAST_MAX_WARPS = 3072;
-// Level-0 compressor, a CTA per block (compress_cta.cu): every block of a
+// Compressor, a CTA per block (compress_cta.cu): every block of a
 // stream whose shape compress_cta_ok takes, the shortened last one too.
 // a.slots holds two staging slots for each of max_ctas CTAs.
 bool compress_cta_ok(uint32_t es, uint32_t B);
@@ -131,6 +119,8 @@ uint32_t compress_cta_max(uint32_t S, uint32_t sms);   // CTAs that can be resid
 size_t compress_cta_slots_bytes(uint32_t S, uint32_t ctas);
 cudaError_t launch_compress_cta(const CodecArgs &a, uint32_t max_ctas, cudaStream_t s);
 // its parts, by translation unit
+cudaError_t launch_compress_cta_l1(const CodecArgs &a, uint32_t max_ctas, cudaStream_t s);
+cudaError_t launch_compress_cta_l1_vis(const CodecArgs &a, uint32_t max_ctas, cudaStream_t s);
 cudaError_t launch_compress_cta1(const CodecArgs &a, uint32_t max_ctas, cudaStream_t s);
 cudaError_t launch_compress_cta2(const CodecArgs &a, uint32_t max_ctas, cudaStream_t s);
 cudaError_t launch_compress_cta8(const CodecArgs &a, uint32_t max_ctas, cudaStream_t s);

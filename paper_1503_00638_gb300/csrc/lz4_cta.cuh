@@ -1,7 +1,7 @@
-// Level-0 LZ4 block encoder for a CTA of W warps (Sec. 4.1, 4.2.1): the same
-// greedy parse, byte for byte, as lz4_encode_bitmap and
-// lz4_encode_bitmap_fast (lz4_warp.cuh has the format and the parse graph),
-// for blocks of up to 64 KiB.
+// LZ4 block encoder for a CTA of W warps (Sec. 4.1, 4.2.1), for blocks of up to
+// 64 KiB: at level 0 the same greedy parse, byte for byte, as
+// lz4_encode_bitmap and lz4_encode_bitmap_fast (lz4_warp.cuh has the format
+// and the parse graph), at level 1 that of lz4_encode_warp.
 //
 // Why a CTA and not a warp: the block is the unit that shared memory holds,
 // so one warp per block leaves an SM with as many warps as blocks fit (20 at
@@ -10,7 +10,7 @@
 // warps per SM at 64 registers for every block size, each thread holding one
 // 32-word group of the bit transpose.
 //
-// The stages, a barrier between each:
+// The stages of level 0, a barrier between each:
 //   1. word-equality bitmaps E[k] = {row, run} (the caller, or
 //      cta_eq_bitmaps from shared memory);
 //   2. thread u derives the candidates of bitmap word u, their run ends and,
@@ -26,6 +26,10 @@
 //      largest part of the one-warp encoder's instructions; a list of 4-byte
 //      words still took 1140 of a CHIME-shaped block's 5070 warp
 //      instructions).
+// At level 1 the search is a chain (where it probes depends on what it found):
+// the first warp searches (lz4_next_match) for a descriptor per thread, then
+// stages 5 and 6 write those sequences, instead of one sequence after another
+// by the warp that searches.
 #pragma once
 
 #include "lz4_warp.cuh"
@@ -68,33 +72,47 @@ struct CtaScratch {
     uint32_t *row;    // bit-row candidates
     uint32_t *pre;    // run ends before a bitmap word: bit-row | run << 16
     uint2 *node;      // {position, first candidate | successor << 16}
-    uint2 *desc;      // sequence descriptors, then the literal list's entries
+    uint2 *desc;      // sequences {match start | offset << 16, match end}, then the
+                      // literal list's entries
     uint32_t *ex;     // exchange words between the warps (EX_*)
+    uint16_t *table;  // level 1: the hash table (2^hbits entries), the rest but
+                      // desc and ex unused
     uint16_t *jmp;    // jump tables: over E, cer and ceu, dead by then
 };
 enum : uint32_t { EX_NZ = 0, EX_CNT = 16, EX_SCAN = 32, EX_LIT = 48, EX_CTL = 64, EX_WORDS = 72 };
 
-__host__ __device__ constexpr uint32_t cta_scratch_bytes(uint32_t W)
+// Hash bits of level 1 for blocks of S bytes.
+__host__ __device__ constexpr uint32_t cta_hbits(uint32_t S) { return S <= 8192u ? 11u : S <= 16384u ? 12u : 13u; }
+
+template <int LEVEL>
+__host__ __device__ constexpr uint32_t cta_scratch_bytes(uint32_t W, uint32_t hbits = 0)
 {
-    return 4u * (2u * (32u * W + 1u) + 5u * 32u * W + 2u * cta_node_cap(W) + 2u * (32u * W + 1u) +
-                 EX_WORDS);
+    return LEVEL >= 1 ? (2u << hbits) + 4u * (2u * (32u * W + 1u) + EX_WORDS)
+                      : 4u * (2u * (32u * W + 1u) + 5u * 32u * W + 2u * cta_node_cap(W) +
+                              2u * (32u * W + 1u) + EX_WORDS);
 }
 
-BSG_D CtaScratch cta_scratch(uint8_t *base, uint32_t W)
+template <int LEVEL>
+BSG_D CtaScratch cta_scratch(uint8_t *base, uint32_t W, uint32_t hbits = 0)
 {
-    CtaScratch c;
-    uint32_t *p = reinterpret_cast<uint32_t *>(base);   // 8-byte aligned
-    c.E = reinterpret_cast<uint2 *>(p);
-    c.jmp = reinterpret_cast<uint16_t *>(p);
-    p += 2u * (32u * W + 1u);
-    c.cer = p;
-    c.ceu = p + 32u * W;
-    c.any = p + 64u * W;
-    c.row = p + 96u * W;
-    c.pre = p + 128u * W;
-    p += 160u * W;
-    c.node = reinterpret_cast<uint2 *>(p);
-    p += 2u * cta_node_cap(W);
+    CtaScratch c{};
+    uint32_t *p = reinterpret_cast<uint32_t *>(base);   // 16-byte aligned
+    if (LEVEL >= 1) {
+        c.table = reinterpret_cast<uint16_t *>(p);
+        p += (2u << hbits) / 4u;
+    } else {
+        c.E = reinterpret_cast<uint2 *>(p);
+        c.jmp = reinterpret_cast<uint16_t *>(p);
+        p += 2u * (32u * W + 1u);
+        c.cer = p;
+        c.ceu = p + 32u * W;
+        c.any = p + 64u * W;
+        c.row = p + 96u * W;
+        c.pre = p + 128u * W;
+        p += 160u * W;
+        c.node = reinterpret_cast<uint2 *>(p);
+        p += 2u * cta_node_cap(W);
+    }
     c.desc = reinterpret_cast<uint2 *>(p);
     p += 2u * (32u * W + 1u);
     c.ex = p;
@@ -155,9 +173,11 @@ BSG_D uint32_t cta_first_set(const CtaScratch &c, uint32_t from, uint32_t to, ui
 // before the literal runs are copied; idle() once by the last warp, when
 // there is more than one, while the first alone walks the parse graph.
 // Returns the size; the caller's next barrier ends the reads of src.
-template <class SizeKnown, class Idle>
+// (Level 1: c.E is not used; hbits as cta_hbits of the stream's full blocks.)
+template <int LEVEL, class SizeKnown, class Idle>
 BSG_D uint32_t cta_lz4_encode(const uint8_t *src, uint32_t S, uint32_t rowlen, uint8_t *dst,
-                              const CtaScratch &c, uint32_t W, SizeKnown size_known, Idle idle)
+                              const CtaScratch &c, uint32_t W, uint32_t hbits, SizeKnown size_known,
+                              Idle idle)
 {
     const uint32_t tid = fresh_tid(), lane = tid & 31u, warp = tid >> 5, NT = 32u * W;
     const uint32_t *s32 = reinterpret_cast<const uint32_t *>(src);
@@ -165,89 +185,99 @@ BSG_D uint32_t cta_lz4_encode(const uint8_t *src, uint32_t S, uint32_t rowlen, u
     const uint32_t R = (rowlen & 3u) ? 0u : rowlen / 4u;
     const uint32_t cap_nodes = cta_node_cap(W);
 
-    // candidates: bits w, w + 1 and w + 2 set; a run of candidates ends where
-    // the next bit is no candidate
-    uint32_t cer = 0, ceu = 0, nz;
-    {
-        uint32_t crow = 0, crun = 0;
-        if (tid < NB) {
-            static_assert(LZ4_L0_MINWORDS == 3, "candidate masks");
-            const uint2 e = c.E[tid], n = tid + 1u < NB ? c.E[tid + 1u] : make_uint2(0u, 0u);
-            crow = e.x & funnel_r(e.x, n.x, 1u) & funnel_r(e.x, n.x, 2u);
-            crun = e.y & funnel_r(e.y, n.y, 1u) & funnel_r(e.y, n.y, 2u);
-            cer = crow & ~funnel_r(crow, (n.x & 7u) == 7u ? 1u : 0u, 1u);
-            ceu = crun & ~funnel_r(crun, (n.y & 7u) == 7u ? 1u : 0u, 1u);
-        }
-        c.cer[tid] = cer;
-        c.ceu[tid] = ceu;
-        c.any[tid] = crow | crun;
-        c.row[tid] = crow;
-        nz = __ballot_sync(FULL, (crow | crun) != 0u);
-    }
-    const uint32_t cnt = (uint32_t)__popc(cer) | ((uint32_t)__popc(ceu) << 16);
-    uint32_t incl = cnt;
-#pragma unroll
-    for (int d = 1; d < 32; d <<= 1) {
-        const uint32_t t = __shfl_up_sync(FULL, incl, d);
-        if (lane >= (uint32_t)d) incl += t;
-    }
-    if (lane == 31) {
-        c.ex[EX_NZ + warp] = nz;
-        c.ex[EX_CNT + warp] = incl;
-    }
-    __syncthreads();
-    uint32_t tot = 0, rank = incl - cnt;
-#pragma unroll 1
-    for (uint32_t j = 0; j < W; j++) {
-        const uint32_t t = c.ex[EX_CNT + j];
-        if (j < warp) rank += t;
-        tot += t;
-    }
-    const uint32_t Nr = tot & 0xffffu, N = Nr + (tot >> 16);
-    const bool some = S >= LZ4_MFLIMIT + 1u && S >= LZ4_LASTLITERALS + LZ4_L0_MINMATCH;
+    const bool some = LEVEL >= 1 || (S >= LZ4_MFLIMIT + 1u && S >= LZ4_LASTLITERALS + LZ4_L0_MINMATCH);
     const uint32_t wlim = some ? (S - LZ4_LASTLITERALS - LZ4_L0_MINMATCH) / 4u : 0u;
     const uint32_t matchlimit = S - LZ4_LASTLITERALS, cap = matchlimit / 4u;
-    const bool graph = some && N < cap_nodes;   // nodes 0 .. N - 1 and the start, N
-    if (graph) {
-        // node ids in position order within each kind, bit-row kind first
-        c.pre[tid] = rank;
-        uint32_t id = rank & 0xffffu;
-#pragma unroll 1
-        for (uint32_t m = cer; m; m &= m - 1u) c.node[id++].x = 32u * tid + (uint32_t)(__ffs(m) - 1);
-        id = Nr + (rank >> 16);
-#pragma unroll 1
-        for (uint32_t m = ceu; m; m &= m - 1u) c.node[id++].x = 32u * tid + (uint32_t)(__ffs(m) - 1);
-    }
-    __syncthreads();
-    if (graph) {
-#pragma unroll 1
-        for (uint32_t id = tid; id <= N; id += NT) {
-            uint32_t p = 0;
-            if (id < N) {
-                uint32_t e = c.node[id].x + LZ4_L0_MINWORDS;
-                if (e > cap) e = cap;
-                p = 4u * e;
-                if (p < matchlimit) {
-                    const uint32_t x = s32[e] ^ s32[e - (id < Nr ? R : 1u)];
-                    uint32_t eq = x ? ((uint32_t)(__ffs(x) - 1) >> 3) : 4u;
-                    if (eq > matchlimit - p) eq = matchlimit - p;
-                    p += eq;
-                }
+    uint32_t N = 0, Nr = 0;   // nodes of the parse graph, those of the bit-row kind first
+    bool graph = false;
+    Lz4Probe probe;
+    if (LEVEL >= 1) {
+        uint4 *t4 = reinterpret_cast<uint4 *>(c.table);
+        for (uint32_t i = tid; i < (2u << hbits) / 16u; i += NT) t4[i] = make_uint4(0u, 0u, 0u, 0u);
+        __syncthreads();
+    } else {
+        // candidates: bits w, w + 1 and w + 2 set; a run of candidates ends where
+        // the next bit is no candidate
+        uint32_t cer = 0, ceu = 0, nz;
+        {
+            uint32_t crow = 0, crun = 0;
+            if (tid < NB) {
+                static_assert(LZ4_L0_MINWORDS == 3, "candidate masks");
+                const uint2 e = c.E[tid], n = tid + 1u < NB ? c.E[tid + 1u] : make_uint2(0u, 0u);
+                crow = e.x & funnel_r(e.x, n.x, 1u) & funnel_r(e.x, n.x, 2u);
+                crun = e.y & funnel_r(e.y, n.y, 1u) & funnel_r(e.y, n.y, 2u);
+                cer = crow & ~funnel_r(crow, (n.x & 7u) == 7u ? 1u : 0u, 1u);
+                ceu = crun & ~funnel_r(crun, (n.y & 7u) == 7u ? 1u : 0u, 1u);
             }
-            const uint32_t w = cta_first_set(c, (p + 3u) / 4u, wlim, W);
-            uint32_t succ = CTA_NONE << 16;
-            if (w != ~0u) {
-                // the previous bit-row wins a tie
-                const uint32_t wd = w >> 5, below = (1u << (w & 31u)) - 1u;
-                const bool row = (c.row[wd] >> (w & 31u)) & 1u;
-                const uint32_t nx = row ? (c.pre[wd] & 0xffffu) + (uint32_t)__popc(c.cer[wd] & below)
-                                        : Nr + (c.pre[wd] >> 16) + (uint32_t)__popc(c.ceu[wd] & below);
-                succ = w | (nx << 16);
-            }
-            c.node[id] = make_uint2(p, succ);
+            c.cer[tid] = cer;
+            c.ceu[tid] = ceu;
+            c.any[tid] = crow | crun;
+            c.row[tid] = crow;
+            nz = __ballot_sync(FULL, (crow | crun) != 0u);
         }
+        const uint32_t cnt = (uint32_t)__popc(cer) | ((uint32_t)__popc(ceu) << 16);
+        uint32_t incl = cnt;
+#pragma unroll
+        for (int d = 1; d < 32; d <<= 1) {
+            const uint32_t t = __shfl_up_sync(FULL, incl, d);
+            if (lane >= (uint32_t)d) incl += t;
+        }
+        if (lane == 31) {
+            c.ex[EX_NZ + warp] = nz;
+            c.ex[EX_CNT + warp] = incl;
+        }
+        __syncthreads();
+        uint32_t tot = 0, rank = incl - cnt;
+#pragma unroll 1
+        for (uint32_t j = 0; j < W; j++) {
+            const uint32_t t = c.ex[EX_CNT + j];
+            if (j < warp) rank += t;
+            tot += t;
+        }
+        Nr = tot & 0xffffu;
+        N = Nr + (tot >> 16);
+        graph = some && N < cap_nodes;   // nodes 0 .. N - 1 and the start, N
+        if (graph) {
+            // node ids in position order within each kind, bit-row kind first
+            c.pre[tid] = rank;
+            uint32_t id = rank & 0xffffu;
+#pragma unroll 1
+            for (uint32_t m = cer; m; m &= m - 1u) c.node[id++].x = 32u * tid + (uint32_t)(__ffs(m) - 1);
+            id = Nr + (rank >> 16);
+#pragma unroll 1
+            for (uint32_t m = ceu; m; m &= m - 1u) c.node[id++].x = 32u * tid + (uint32_t)(__ffs(m) - 1);
+        }
+        __syncthreads();
+        if (graph) {
+#pragma unroll 1
+            for (uint32_t id = tid; id <= N; id += NT) {
+                uint32_t p = 0;
+                if (id < N) {
+                    uint32_t e = c.node[id].x + LZ4_L0_MINWORDS;
+                    if (e > cap) e = cap;
+                    p = 4u * e;
+                    if (p < matchlimit) {
+                        const uint32_t x = s32[e] ^ s32[e - (id < Nr ? R : 1u)];
+                        uint32_t eq = x ? ((uint32_t)(__ffs(x) - 1) >> 3) : 4u;
+                        if (eq > matchlimit - p) eq = matchlimit - p;
+                        p += eq;
+                    }
+                }
+                const uint32_t w = cta_first_set(c, (p + 3u) / 4u, wlim, W);
+                uint32_t succ = CTA_NONE << 16;
+                if (w != ~0u) {
+                    // the previous bit-row wins a tie
+                    const uint32_t wd = w >> 5, below = (1u << (w & 31u)) - 1u;
+                    const bool row = (c.row[wd] >> (w & 31u)) & 1u;
+                    const uint32_t nx = row ? (c.pre[wd] & 0xffffu) + (uint32_t)__popc(c.cer[wd] & below)
+                                            : Nr + (c.pre[wd] >> 16) + (uint32_t)__popc(c.ceu[wd] & below);
+                    succ = w | (nx << 16);
+                }
+                c.node[id] = make_uint2(p, succ);
+            }
+        }
+        __syncthreads();
     }
-    __syncthreads();
     uint32_t x0 = N, pos = 0;   // warp 0: where the next descriptors start
     bool more = some;
     if (W > 1 && warp == W - 1u) idle();
@@ -275,7 +305,15 @@ BSG_D uint32_t cta_lz4_encode(const uint8_t *src, uint32_t S, uint32_t rowlen, u
     for (;;) {
         if (warp == 0) {
             uint32_t n = 0;
-            if (graph) {
+            if (LEVEL >= 1) {
+#pragma unroll 1
+                for (; more && n < NT; n++) {
+                    uint32_t mp, off, len;
+                    more = lz4_next_match<1>(src, S, rowlen, c.table, hbits, probe, lane, mp, off, len);
+                    if (!more) break;
+                    if (lane == 0) c.desc[n] = make_uint2(mp | (off << 16), mp + len);
+                }
+            } else if (graph) {
 #pragma unroll 1
                 while (more && n < NT) {
                     // lane k: the node k steps after x0 and the node after it
@@ -287,8 +325,8 @@ BSG_D uint32_t cta_lz4_encode(const uint8_t *src, uint32_t S, uint32_t rowlen, u
                     const uint32_t succ = x != CTA_NONE ? c.node[x].y : CTA_NONE << 16;
                     const uint32_t nx = succ >> 16;
                     if (nx != CTA_NONE)
-                        c.desc[n + lane] = make_uint2(4u * (succ & 0xffffu) | (nx < Nr ? 1u << 31 : 0u),
-                                                      c.node[nx].x);
+                        c.desc[n + lane] =
+                            make_uint2(4u * (succ & 0xffffu) | ((nx < Nr ? rowlen : 4u) << 16), c.node[nx].x);
                     const uint32_t got = (uint32_t)__popc(__ballot_sync(FULL, nx != CTA_NONE));
                     x0 = __shfl_sync(FULL, nx, 31);
                     n += got;
@@ -315,7 +353,7 @@ BSG_D uint32_t cta_lz4_encode(const uint8_t *src, uint32_t S, uint32_t rowlen, u
                         if (eq > matchlimit - pos) eq = matchlimit - pos;
                         pos += eq;
                     }
-                    if (lane == 0) c.desc[n] = make_uint2(4u * w | (row ? 1u << 31 : 0u), pos);
+                    if (lane == 0) c.desc[n] = make_uint2(4u * w | ((row ? rowlen : 4u) << 16), pos);
                 }
             }
             if (lane == 0) {
@@ -336,10 +374,10 @@ BSG_D uint32_t cta_lz4_encode(const uint8_t *src, uint32_t S, uint32_t rowlen, u
             mp = last ? S : anchor;
             if (mine) {
                 const uint2 q = c.desc[tid];
-                off = (q.x >> 31) ? rowlen : 4u;
-                mp = q.x & 0x7fffffffu;
+                off = q.x >> 16;
+                mp = q.x & 0xffffu;
                 // back up over up to 3 equal bytes (never before the literal anchor)
-                if (mp > anchor && mp > off) {
+                if (LEVEL == 0 && mp > anchor && mp > off) {
                     const uint32_t x = ld32u(src, mp - 4u) ^ ld32u(src, mp - 4u - off);
                     uint32_t back = (x ? (uint32_t)__clz(x) : 32u) >> 3;
                     if (back > 3u) back = 3u;

@@ -256,9 +256,15 @@ BSG_D uint32_t lz4_emit_last(uint8_t *dst, uint32_t o, const uint8_t *src, uint3
     return o + 1 + nll + LL;
 }
 
-// Encode src[0, S) (word aligned, readable up to S + 8) into dst (capacity
-// lz4_bound(S)), taking only matches of at least LZ4_MINMATCH_OF<LEVEL>
-// bytes.
+// The match search of the probing encoder: where it stands in a block.
+struct Lz4Probe {
+    uint32_t pos = 0, fails = 0, it = 0;
+    uint32_t anchor = 0;   // end of the last match
+};
+
+// Next match of the probing search, for one warp; false when there is none
+// (or the progress guard tripped, which valid sizes cannot do).  Matches have
+// at least LZ4_MINMATCH_OF<LEVEL> bytes.
 //
 // Each step probes 32 word-aligned positions p at once.  Candidates:
 //  * the same column of the previous bit-row, p - rowlen (a bit-row repeating
@@ -271,115 +277,132 @@ BSG_D uint32_t lz4_emit_last(uint8_t *dst, uint32_t o, const uint8_t *src, uint3
 //    after LZ4_ACCEL_WINDOWS fruitless steps the probe stride doubles (to 16
 //    bytes at most).
 // The first position whose candidate agrees on the minimum match is taken,
-// extended back by up to 3 bytes and forward warp-wide.  Returns the compressed size,
-// or 0xffffffff if the progress guard tripped (cannot happen for valid sizes).
+// extended back by up to 3 bytes and forward warp-wide.
+template <int LEVEL>
+BSG_D bool lz4_next_match(const uint8_t *src, uint32_t S, uint32_t rowlen, uint16_t *table,
+                          uint32_t hbits, Lz4Probe &q, uint32_t lane, uint32_t &mp_out,
+                          uint32_t &off_out, uint32_t &len_out)
+{
+    const uint32_t lt = lanemask_lt();
+    const uint32_t le = lt | (1u << lane);
+    const uint32_t *s32 = reinterpret_cast<const uint32_t *>(src);
+    if (rowlen & 3u) rowlen = 0;
+    if (S < LZ4_MFLIMIT + 1 || S < LZ4_LASTLITERALS + LZ4_MINMATCH_OF<LEVEL>) return false;
+    // a probe at p verifies MM bytes, so it must end by the match-end
+    // bound (p + MM <= S - 5), which is also below the last allowed match start
+    constexpr uint32_t MM = LZ4_MINMATCH_OF<LEVEL>;
+    const uint32_t mflimit = S - LZ4_LASTLITERALS - MM;
+    const uint32_t matchlimit = S - LZ4_LASTLITERALS;  // match end bound
+    const uint32_t guard = S / 4 + 8;
+    while (q.pos <= mflimit) {
+        if (++q.it > guard) return false;
+        uint32_t step = 4;
+        if (LEVEL >= 1) {
+            const uint32_t sh = q.fails / LZ4_ACCEL_WINDOWS;
+            step = 4u << (sh < 2 ? sh : 2);
+        }
+        const uint32_t p = q.pos + step * lane;
+        const bool valid = p <= mflimit;
+        const uint32_t wi = p >> 2;
+        const uint32_t w0 = valid ? s32[wi] : 0u;
+        const uint32_t w1 = valid ? s32[wi + 1] : 0u;
+        static_assert(MM == 8 || MM == 12, "probes verify two or three words");
+        const uint32_t w2 = (MM > 8 && valid) ? s32[wi + 2] : 0u;
+        uint32_t off = 0;
+        if (valid && rowlen && p >= rowlen) {
+            const uint32_t ri = (p - rowlen) >> 2;
+            if (s32[ri] == w0 && s32[ri + 1] == w1 && (MM <= 8 || s32[ri + 2] == w2))
+                off = rowlen;
+        }
+        if (valid && off == 0 && p >= 4 && w1 == w0 && (MM <= 8 || w2 == w0) &&
+            s32[wi - 1] == w0)
+            off = 4;
+        if (LEVEL >= 1) {
+            const uint32_t h = (w0 * 2654435761u) >> (32 - hbits);
+            const uint32_t grp = __match_any_sync(FULL, valid ? h : 0x80000000u);
+            const uint32_t lower = grp & lt;
+            int32_t cand = valid ? (int32_t)table[h] * 4 - 4 : -1;
+            if (valid && lower) cand = (int32_t)(q.pos + step * (31 - __clz(lower)));
+            if (valid && off == 0 && cand >= 0 && s32[cand >> 2] == w0 &&
+                s32[(cand >> 2) + 1] == w1)
+                off = p - (uint32_t)cand;
+            const uint32_t mm0 = __ballot_sync(FULL, off != 0);
+            const uint32_t vm = __ballot_sync(FULL, valid);
+            // insert the probed positions up to the match (all of them if none)
+            const uint32_t upto = mm0 ? ((2u << (__ffs(mm0) - 1)) - 1u) : FULL;
+            const uint32_t mine = grp & upto & vm;
+            if (valid && (upto >> lane & 1u) && (mine & ~le) == 0)
+                table[h] = (uint16_t)((p >> 2) + 1);
+            __syncwarp();
+        }
+        const uint32_t mm = __ballot_sync(FULL, off != 0);
+        if (mm == 0) {
+            q.fails++;
+            q.pos += step * 32;
+            continue;
+        }
+        const uint32_t fl = __ffs(mm) - 1;
+        const uint32_t p0 = q.pos + step * fl;
+        const uint32_t moff = __shfl_sync(FULL, off, fl);
+        uint32_t mp = p0;
+        // back up over up to 3 equal bytes (never before the literal anchor)
+#pragma unroll
+        for (int b = 0; b < 3; b++) {
+            if (mp > q.anchor && mp > moff && src[mp - 1] == src[mp - 1 - moff]) mp--;
+        }
+        const uint32_t mc = mp - moff;
+        uint32_t len = p0 + MM - mp;   // the verified bytes, and the backed-up ones
+        // extend forward, 128 bytes per step
+        for (uint32_t g2 = 0; g2 < S; g2 += 128) {
+            const uint32_t x0 = mp + len + 4 * lane;
+            const int room = (int)matchlimit - (int)x0;
+            uint32_t eq = 0;
+            if (room > 0) {
+                const uint32_t x = ld32u(src, x0) ^ ld32u(src, mc + len + 4 * lane);
+                eq = x ? ((uint32_t)(__ffs(x) - 1) >> 3) : 4u;
+                if ((int)eq > room) eq = (uint32_t)room;
+            }
+            const uint32_t stop = __ballot_sync(FULL, eq < 4);
+            if (stop == 0) {
+                len += 128;
+                continue;
+            }
+            const uint32_t sl = __ffs(stop) - 1;
+            len += 4 * sl + __shfl_sync(FULL, eq, sl);
+            break;
+        }
+        mp_out = mp;
+        off_out = moff;
+        len_out = len;
+        q.anchor = mp + len;
+        q.pos = (q.anchor + 3u) & ~3u;
+        q.fails = 0;
+        return true;
+    }
+    return false;
+}
+
+// Encode src[0, S) (word aligned, readable up to S + 8) into dst (capacity
+// lz4_bound(S)) by one warp with the matches of lz4_next_match.  Returns the
+// compressed size, or 0xffffffff if the progress guard tripped (cannot happen
+// for valid sizes).
 template <int LEVEL, int HBITS>
 BSG_D uint32_t lz4_encode_warp(const uint8_t *src, uint32_t S, uint32_t rowlen, uint8_t *dst,
                                uint16_t *table)
 {
     const uint32_t lane = threadIdx.x & 31u;
-    const uint32_t lt = lanemask_lt();
-    const uint32_t le = lt | (1u << lane);
-    const uint32_t *s32 = reinterpret_cast<const uint32_t *>(src);
     if (LEVEL >= 1) {
         uint4 *t4 = reinterpret_cast<uint4 *>(table);
         for (uint32_t i = lane; i < (2u << HBITS) / 16u; i += 32) t4[i] = make_uint4(0, 0, 0, 0);
         __syncwarp();
     }
-    if (rowlen & 3u) rowlen = 0;
-    uint32_t anchor = 0, o = 0;
-    if (S >= LZ4_MFLIMIT + 1 && S >= LZ4_LASTLITERALS + LZ4_MINMATCH_OF<LEVEL>) {
-        // a probe at p verifies MM bytes, so it must end by the match-end
-        // bound (p + MM <= S - 5), which is also below the last allowed match start
-        constexpr uint32_t MM = LZ4_MINMATCH_OF<LEVEL>;
-        const uint32_t mflimit = S - LZ4_LASTLITERALS - MM;
-        const uint32_t matchlimit = S - LZ4_LASTLITERALS;  // match end bound
-        uint32_t pos = 0, fails = 0;
-        const uint32_t guard = S / 4 + 8;
-        uint32_t it = 0;
-        while (pos <= mflimit) {
-            if (++it > guard) return 0xffffffffu;
-            uint32_t step = 4;
-            if (LEVEL >= 1) {
-                const uint32_t sh = fails / LZ4_ACCEL_WINDOWS;
-                step = 4u << (sh < 2 ? sh : 2);
-            }
-            const uint32_t p = pos + step * lane;
-            const bool valid = p <= mflimit;
-            const uint32_t wi = p >> 2;
-            const uint32_t w0 = valid ? s32[wi] : 0u;
-            const uint32_t w1 = valid ? s32[wi + 1] : 0u;
-            static_assert(MM == 8 || MM == 12, "probes verify two or three words");
-            const uint32_t w2 = (MM > 8 && valid) ? s32[wi + 2] : 0u;
-            uint32_t off = 0;
-            if (valid && rowlen && p >= rowlen) {
-                const uint32_t ri = (p - rowlen) >> 2;
-                if (s32[ri] == w0 && s32[ri + 1] == w1 && (MM <= 8 || s32[ri + 2] == w2))
-                    off = rowlen;
-            }
-            if (valid && off == 0 && p >= 4 && w1 == w0 && (MM <= 8 || w2 == w0) &&
-                s32[wi - 1] == w0)
-                off = 4;
-            if (LEVEL >= 1) {
-                const uint32_t h = (w0 * 2654435761u) >> (32 - HBITS);
-                const uint32_t grp = __match_any_sync(FULL, valid ? h : 0x80000000u);
-                const uint32_t lower = grp & lt;
-                int32_t cand = valid ? (int32_t)table[h] * 4 - 4 : -1;
-                if (valid && lower) cand = (int32_t)(pos + step * (31 - __clz(lower)));
-                if (valid && off == 0 && cand >= 0 && s32[cand >> 2] == w0 &&
-                    s32[(cand >> 2) + 1] == w1)
-                    off = p - (uint32_t)cand;
-                const uint32_t mm0 = __ballot_sync(FULL, off != 0);
-                const uint32_t vm = __ballot_sync(FULL, valid);
-                // insert the probed positions up to the match (all of them if none)
-                const uint32_t upto = mm0 ? ((2u << (__ffs(mm0) - 1)) - 1u) : FULL;
-                const uint32_t mine = grp & upto & vm;
-                if (valid && (upto >> lane & 1u) && (mine & ~le) == 0)
-                    table[h] = (uint16_t)((p >> 2) + 1);
-                __syncwarp();
-            }
-            const uint32_t mm = __ballot_sync(FULL, off != 0);
-            if (mm == 0) {
-                fails++;
-                pos += step * 32;
-                continue;
-            }
-            const uint32_t fl = __ffs(mm) - 1;
-            const uint32_t p0 = pos + step * fl;
-            const uint32_t moff = __shfl_sync(FULL, off, fl);
-            uint32_t mp = p0;
-            // back up over up to 3 equal bytes (never before the literal anchor)
-#pragma unroll
-            for (int b = 0; b < 3; b++) {
-                if (mp > anchor && mp > moff && src[mp - 1] == src[mp - 1 - moff]) mp--;
-            }
-            const uint32_t mc = mp - moff;
-            uint32_t len = p0 + MM - mp;   // the verified bytes, and the backed-up ones
-            // extend forward, 128 bytes per step
-            for (uint32_t g2 = 0; g2 < S; g2 += 128) {
-                const uint32_t q = mp + len + 4 * lane;
-                const int room = (int)matchlimit - (int)q;
-                uint32_t eq = 0;
-                if (room > 0) {
-                    const uint32_t x = ld32u(src, q) ^ ld32u(src, mc + len + 4 * lane);
-                    eq = x ? ((uint32_t)(__ffs(x) - 1) >> 3) : 4u;
-                    if ((int)eq > room) eq = (uint32_t)room;
-                }
-                const uint32_t stop = __ballot_sync(FULL, eq < 4);
-                if (stop == 0) {
-                    len += 128;
-                    continue;
-                }
-                const uint32_t sl = __ffs(stop) - 1;
-                len += 4 * sl + __shfl_sync(FULL, eq, sl);
-                break;
-            }
-            o = lz4_emit(dst, o, src, anchor, mp, moff, len, lane);
-            anchor = mp + len;
-            pos = (anchor + 3u) & ~3u;
-            fails = 0;
-        }
+    Lz4Probe q;
+    uint32_t anchor = 0, o = 0, mp, off, len;
+    while (lz4_next_match<LEVEL>(src, S, rowlen, table, HBITS, q, lane, mp, off, len)) {
+        o = lz4_emit(dst, o, src, anchor, mp, off, len, lane);
+        anchor = mp + len;
     }
+    if (q.it > S / 4 + 8) return 0xffffffffu;
     o = lz4_emit_last(dst, o, src, anchor, S, lane);
     __syncwarp();
     return o;

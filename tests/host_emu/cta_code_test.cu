@@ -80,7 +80,8 @@ int main(int argc, char **argv)
     memcpy(buf, x.data(), S);
     memset(out, 0, sizeof out);
     memset(scr, 0x5A, sizeof scr);
-    if (cta_scratch_bytes(W) > sizeof scr) return 3;
+    const uint32_t hbits = cta_hbits(S);
+    if (cta_scratch_bytes<0>(W) > sizeof scr || cta_scratch_bytes<1>(W, hbits) > sizeof scr) return 3;
     uint32_t cs = 0, known = 0;
     uint8_t *enc = out + 4;   // the slot's four length bytes come first
     run_cta(32 * W, [&] {
@@ -90,10 +91,10 @@ int main(int argc, char **argv)
         case 4: transpose<4>(Bb); break;
         default: transpose<8>(Bb); break;
         }
-        const CtaScratch c = cta_scratch(scr, W);
+        const CtaScratch c = cta_scratch<0>(scr, W);
         cta_eq_bitmaps(reinterpret_cast<const uint32_t *>(buf), S / 4, (rowlen & 3u) ? 0u : rowlen / 4, c, W);
         __syncthreads();
-        const uint32_t o = cta_lz4_encode(buf, S, rowlen, enc, c, W, [&](uint32_t s) {
+        const uint32_t o = cta_lz4_encode<0>(buf, S, rowlen, enc, c, W, hbits, [&](uint32_t s) {
             if (threadIdx.x == 0) known = s;
         }, [] {});
         if (threadIdx.x == 0) cs = o;
@@ -112,6 +113,25 @@ int main(int argc, char **argv)
     }
     if (orc_lz4_decompress_block(enc, cs, back.data(), S) || memcmp(back.data(), rows.data(), S)) {
         fprintf(stderr, "the oracle rejects the block\n");
+        return 1;
+    }
+    // level 1 against the one-warp encoder's search and emission
+    alignas(16) static uint8_t out1[70000];
+    uint32_t cs1 = 0;
+    const uint32_t W1 = (S + 8191) / 8192;
+    run_cta(32 * W1, [&] {
+        const CtaScratch c = cta_scratch<1>(scr, W1, hbits);
+        const uint32_t o = cta_lz4_encode<1>(buf, S, rowlen, out1 + 4, c, W1, hbits, [](uint32_t) {}, [] {});
+        if (threadIdx.x == 0) cs1 = o;
+    });
+    run_cta(32, [&] {
+        const uint32_t o = hbits == 11   ? lz4_encode_warp<1, 11>(buf, S, rowlen, ref, (uint16_t *)bm)
+                           : hbits == 12 ? lz4_encode_warp<1, 12>(buf, S, rowlen, ref, (uint16_t *)bm)
+                                         : lz4_encode_warp<1, 13>(buf, S, rowlen, ref, (uint16_t *)bm);
+        if (threadIdx.x == 0) want = o;
+    });
+    if (cs1 != want || memcmp(out1 + 4, ref, cs1)) {
+        fprintf(stderr, "level 1 differs: %u / %u bytes\n", cs1, want);
         return 1;
     }
     std::vector<uint8_t> oc(lz4_bound(S) + 16);

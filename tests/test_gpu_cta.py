@@ -1,4 +1,4 @@
-"""The level-0 compressor (a CTA per block) against the general compressor:
+"""The compressor (a CTA per block) against the general compressor:
 `compress_noalloc` takes the general kernel for every shape, and both must
 write the same bytes; the oracle decodes them.  Sizes: one block and many,
 block sizes of one to sixteen warps and in between, shortened last blocks
@@ -28,17 +28,18 @@ def _walk(n, es, seed, noisy):
                                                       8: np.uint64}[es])
 
 
+@pytest.mark.parametrize("level", [0, 1])
 @pytest.mark.parametrize("noisy", [False, True])
 @pytest.mark.parametrize("es,B", SHAPES)
-def test_streams_equal_the_general_compressors(orc, es, B, noisy):
+def test_streams_equal_the_general_compressors(orc, es, B, noisy, level):
     from paper_1503_00638_gb300 import bsgpu
     many = max(2, 40_000_000 // (B * es * 10))       # more blocks than CTAs for the small blocks
     for n in (8, B - 8 if B > 8 else 8, B, B + 8, 3 * B + 40 + 5, many * B, many * B + B // 2 + 3):
         x = _walk(n, es, n % 1009, noisy)
         d = torch.from_numpy(x.view({1: np.uint8, 2: np.int16, 4: np.int32, 8: np.int64}[es])).cuda()
-        c = bsgpu.compress(d, B)
+        c = bsgpu.compress(d, B, level=level)
         assert bsgpu.status(c.ws) == 0
-        out, nb, offs = bsgpu.compress_noalloc(d, B, offsets=torch.zeros_like(c.offsets))
+        out, nb, offs = bsgpu.compress_noalloc(d, B, offsets=torch.zeros_like(c.offsets), level=level)
         torch.cuda.synchronize()
         assert c.nbytes == int(nb.item())
         assert torch.equal(c.buf[:c.nbytes], out[:c.nbytes])
@@ -83,6 +84,10 @@ def test_cube_streams_equal_rounding_then_compressing(shape, dtype, tslow):
             torch.cuda.synchronize()
             assert c.nbytes == int(nb.item())
             assert torch.equal(c.buf[:c.nbytes], out[:c.nbytes])
+        c = bsgpu.compress_vis_ex(src, cfg.n_samp, cfg.f, compensate=comp, block_elems=2048,
+                                  time_slowest=tslow, level=1)
+        out, nb, _ = bsgpu.compress_noalloc(bits.contiguous(), 2048, elem_size=4, level=1)
+        assert c.nbytes == int(nb.item()) and torch.equal(c.buf[:c.nbytes], out[:c.nbytes])
 
 
 @pytest.mark.parametrize("shape", [(1, 40, 300), (2, 128, 1), (3, 24, 1100), (1, 90, 33)])
