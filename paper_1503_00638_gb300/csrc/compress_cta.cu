@@ -31,7 +31,7 @@ cudaError_t launch_compress_cta(const CodecArgs &a, uint32_t max_ctas, cudaStrea
     switch (a.es) {
     case 1: return launch_compress_cta1(a, max_ctas, s);
     case 2: return launch_compress_cta2(a, max_ctas, s);
-    case 4: return launch_cta_stream<0, 4, CTA_PLAIN, 2048, 1024>(a, max_ctas, s);
+    case 4: return launch_cta_stream<0, 4, CTA_PLAIN, 2048, 1024, 4096, 8192>(a, max_ctas, s);
     default: return launch_compress_cta8(a, max_ctas, s);
     }
 }

@@ -327,15 +327,16 @@ BSG_D uint64_t lookback_some(uint64_t *state, uint32_t tile, uint64_t agg, uint3
 // evenly (CHIME-shaped cube, 256 frequencies, 33024 blocks of 8 KiB: 217 us,
 // issue active 57 %, ALU 54 %, shared-memory pipe 49 %, DRAM 25 %; 24, 28 or
 // 32 warps per SM make no difference).  The one-warp kernel it replaces took
-// 290 us there.  Whole cube, 1.08 GB: 1.10 -> 0.83 ms; 268 MB of float64 in
-// 32 KiB blocks, which took a kernel of two buffers per warp: 0.88 -> 0.20 ms.
+// 290 us there.  Whole cube, 1.08 GB: 1.10 -> 0.86 ms; 268 MB of float64 in
+// 32 KiB blocks, which took a kernel of two buffers per warp: 0.88 -> 0.18 ms.
 //
-// BC: the block size in elements when it is one of the usual ones (4 and
-// 8 KiB; full blocks only), else 0 for any size and for a shortened last
-// block.  With the size known the strides of the bit-rows, the loops over
-// the warps and the tables' places are constants (int32 cube, time slowest, as
-// 8-byte samples in 4 KiB blocks, 127 MB: 279 -> 253 us).  TS: a time-slowest
-// cube.
+// BC: the block size in elements when it is one of the usual ones (4 and 8
+// KiB, 16 and 32 KiB of 4- and 8-byte elements; full blocks only), else 0 for
+// any size and for a shortened last block.  With the size known the strides of
+// the bit-rows, the loops over the warps and the tables' places are constants
+// (int32 cube, time slowest, as 8-byte samples in 4 KiB blocks, 127 MB: 279 ->
+// 253 us; 268 MB of float64 in 32 KiB blocks: 206 -> 182 us).  TS: a
+// time-slowest cube.
 template <int LEVEL, int ES, int MODE, uint32_t BC, bool TS>
 BSG_D void compress_cta_body(const CodecArgs &a)
 {
@@ -477,7 +478,7 @@ BSG_D void compress_cta_body(const CodecArgs &a)
 
 template <int ES, int MODE, uint32_t BC, bool TS>
 __global__ void __launch_bounds__(BC ? 32 * cta_warps(BC *ES) : 32 * CTA_MAX_WARPS,
-                                  BC ? CTA_WARPS_PER_SM / cta_warps(BC *ES) : 2)
+                                  BC ? (cta_warps(BC *ES) > 2 ? 32u : CTA_WARPS_PER_SM) / cta_warps(BC *ES) : 2)
     compress_cta_kernel(const __grid_constant__ CodecArgs a)
 {
     compress_cta_body<0, ES, MODE, BC, TS>(a);
