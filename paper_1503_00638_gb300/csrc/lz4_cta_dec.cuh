@@ -10,8 +10,9 @@
 // more than a barrier per batch, and an SM holds twice the warps for the same
 // shared memory.  In place: a batch's output ends before the input that
 // follows it (the margin that decompress_inplace_kernel's comment derives
-// holds after every sequence), so the matches of one batch never touch what
-// the next one reads.
+// holds after every sequence of a valid block, and the parser ends at the first
+// sequence for which it does not), so the matches of one batch never touch
+// what the next one reads.
 #pragma once
 
 #include "lz4_warp.cuh"
@@ -151,6 +152,10 @@ BSG_D bool cta_lz4_decode(const uint8_t *src, uint32_t ip0, uint32_t clen, uint8
                 // (ML is below 2^31: at most 255 per stream byte)
                 if ((off == 0) | (off > op) | (ML + LZ4_LASTLITERALS > S - op) | (op + LZ4_MFLIMIT > S))
                     break;
+                // (in place: a valid block's output never passes its unread input, by
+                // that margin, so a block whose output does is corrupt, and its
+                // match must not reach what the first warp still reads)
+                if (src == dst && op + ML > ip) break;
                 if (lane == 0) seq[half + n] = make_uint2(op | (off << 16), ML);
                 op += ML;
                 state = 0;
