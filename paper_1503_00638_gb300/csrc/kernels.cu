@@ -737,7 +737,7 @@ __global__ void __launch_bounds__(32, 20) decompress_inplace_kernel(const __grid
             if (cur.eidx != ~0u) comp[cur.eidx] = cur.ebyte;
             __syncwarp();
             good = get_be32(comp + cur.delta) == cur.clen &&
-                   lz4_decode_warp(comp, cur.delta + 4, cur.clen, buf, S) == 0;
+                   lz4_decode_warp(buf, cur.off + cur.delta + 4, cur.clen, buf, S) == 0;
         }
         if (!good && lane == 0) set_status(a.status, BSGPU_ERR_CORRUPT);
         __syncwarp();
@@ -836,7 +836,7 @@ __global__ void __launch_bounds__(32, 20) decompress_inplace_any_kernel(const __
             if (cur.eidx != ~0u) comp[cur.eidx] = cur.ebyte;
             __syncwarp();
             good = get_be32(comp + cur.delta) == cur.clen &&
-                   lz4_decode_warp(comp, cur.delta + 4, cur.clen, buf, S) == 0;
+                   lz4_decode_warp(buf, cur.off + cur.delta + 4, cur.clen, buf, S) == 0;
         }
         if (!good && lane == 0) set_status(a.status, BSGPU_ERR_CORRUPT);
         __syncwarp();

@@ -150,12 +150,10 @@ BSG_D bool cta_lz4_decode(const uint8_t *src, uint32_t ip0, uint32_t clen, uint8
                 }
                 ML += LZ4_MINMATCH;
                 // (ML is below 2^31: at most 255 per stream byte)
-                if ((off == 0) | (off > op) | (ML + LZ4_LASTLITERALS > S - op) | (op + LZ4_MFLIMIT > S))
-                    break;
-                // (in place: a valid block's output never passes its unread input, by
-                // that margin, so a block whose output does is corrupt, and its
-                // match must not reach what the first warp still reads)
-                if (src == dst && op + ML > ip) break;
+                // In place the match must not reach what the parser has still to
+                // read either: by that margin only a corrupt block's would.
+                const uint32_t most = S - LZ4_LASTLITERALS, room = src == dst && ip < most ? ip : most;
+                if ((off == 0) | (off > op) | (op + ML > room) | (op + LZ4_MFLIMIT > S)) break;
                 if (lane == 0) seq[half + n] = make_uint2(op | (off << 16), ML);
                 op += ML;
                 state = 0;

@@ -47,18 +47,21 @@ int main(int argc, char **argv)
             // the sequence that first takes the output past the input is never applied
             const uint32_t read = 4u + ext + (d < 0 ? 0u : 3u * ((uint32_t)d + 1u));
             const bool want = orc_lz4_decompress_block(img.data(), clen, back, S) == 0;
-            memset(D, 0x5A, sizeof D);
-            memcpy(D + ip0, img.data(), clen);
-            bool ok = false;
-            run_cta(64, [&] {
-                const bool r = cta_lz4_decode(D, ip0, clen, D, S, ring, threadIdx.x);
-                if (threadIdx.x == 0) ok = r;
-            });
-            const bool whole = memcmp(D + ip0 + read, img.data() + read, clen - read) == 0;
-            if (want || ok || !whole) {
-                fprintf(stderr, "two warps, match %d bytes behind the input, padding %02x: verdict %d, oracle %d, unread input %s\n",
-                        d, pad, ok, want, whole ? "whole" : "overwritten");
-                return 1;
+            for (int warps : {1, 2}) {
+                memset(D, 0x5A, sizeof D);
+                memcpy(D + ip0, img.data(), clen);
+                bool ok = false;
+                run_cta(32 * warps, [&] {
+                    const bool r = warps == 2 ? cta_lz4_decode(D, ip0, clen, D, S, ring, threadIdx.x)
+                                              : lz4_decode_warp(D, ip0, clen, D, S) == 0;
+                    if (threadIdx.x == 0) ok = r;
+                });
+                const bool whole = memcmp(D + ip0 + read, img.data() + read, clen - read) == 0;
+                if (want || ok || !whole) {
+                    fprintf(stderr, "%d warps, match %d bytes behind the input, padding %02x: verdict %d, oracle %d, unread input %s\n",
+                            warps, d, pad, ok, want, whole ? "whole" : "overwritten");
+                    return 1;
+                }
             }
         }
     printf("ok\n");
