@@ -4,8 +4,10 @@
 // unit test (tests/host_emu/device_code_test.cu) can check them on a CPU.
 #pragma once
 
+#include <cmath>
 #include <cstddef>
 #include <cstdint>
+#include <cstring>
 
 #include "../../include/bsgpu.h"
 
@@ -126,6 +128,43 @@ BSG_HD bool q_usable(uint32_t Q) { return (Q - 0x00800000u) < 0x7f000000u; }
 BSG_HD uint32_t magic_bits(uint32_t Q)   // bit pattern of 2^(k+23)
 {
     return (((Q + 0x007fffffu) >> 24) + 86u) << 23;
+}
+
+BSG_HD uint32_t float_bits(float x)
+{
+#ifdef __CUDA_ARCH__
+    return __float_as_uint(x);
+#else
+    uint32_t u;
+    memcpy(&u, &x, 4);
+    return u;
+#endif
+}
+
+// q of the full covariance in float32: q = fl32(12 f / (N h)), with h = W_ii^2
+// for an auto and 2 (W_ii W_jj +- Re(W_ij^2)) for the real and imaginary parts
+// of a cross product, f12 = 12 f / N.  True when its granularity is beyond
+// doubt: the rounding only asks for the k of 4^k < q, so a quotient that is
+// more than 256 units in the last place (2^-16 of q at least) away from any
+// power of four answers that.  Its error is below 160 units of 2^-24: with
+// |W_ij|^2 <= W_ii W_jj = ww, W_ii W_jj and Re(W_ij^2) carry 3 and 10 units of
+// ww and their sum 2 more, h is more than 0.2 ww, 12 f / N adds one unit and
+// the division four.  All of that supposes normal floats in the middle of the
+// range (where the quick division has its bound too): anything else, and a
+// sum that cancels, is left to the quotient in fp64.
+BSG_HD bool full_q_f32(float f12, float wi, float wj, float wr, float wm, bool is_auto, int part,
+                       float &q)
+{
+    const float ww = wi * wj, re2 = (wr - wm) * (wr + wm);
+    const float h = is_auto ? ww : 2.0f * (part ? ww - re2 : ww + re2);
+#ifdef __CUDA_ARCH__
+    q = __fdividef(f12, h);
+#else
+    q = f12 / h;
+#endif
+    const uint32_t Q = float_bits(q);
+    return fminf(f12, fminf(wi, wj)) > 1e-30f && ww > 1e-30f && ww < 1e30f && h > 0.2f * ww &&
+           q > 1e-30f && q < 1e30f && magic_bits(Q - 256u) == magic_bits(Q + 256u);
 }
 
 #ifdef __CUDACC__

@@ -5,8 +5,6 @@
 // bulk-copy (TMA) engine with the next block prefetched.
 #include <cuda_runtime.h>
 
-#include <cstring>
-
 #include "codec.cuh"
 
 namespace bsg {
@@ -277,24 +275,6 @@ __global__ void __launch_bounds__(256) vis_compensation_end_kernel(float *cft, u
 // (64 per sample) and separate additions.
 BSG_HD uint32_t tri_el(uint32_t r, uint32_t c) { return r * (r + 1) / 2 + c; }
 
-// q = fl32(12 f / h) where h = N2 (ww + re2), N2 = N or 2 N, ww = W_ii W_jj
-// and re2 = +-Re(W_ij^2).  The rounding only asks for the k of 4^k < q: a
-// float32 quotient answers that unless a power of four lies within 256 units
-// in the last place (at least 2^-16 of q; the quotient's error is below 100
-// units of 2^-24: some 18 roundings relative to ww, which h exceeds by 0.2 at
-// least), or the sum cancels, or something leaves the middle of the float
-// range; then the quotient is taken in fp64.
-BSG_HD bool q_beyond_doubt(float q, float ww, float h)
-{
-#ifdef __CUDA_ARCH__
-    const uint32_t Q = __float_as_uint(q);
-#else
-    uint32_t Q;
-    memcpy(&Q, &q, 4);
-#endif
-    return h > 0.2f * ww && q > 1e-30f && q < 1e30f && magic_bits(Q - 256u) == magic_bits(Q + 256u);
-}
-
 __global__ void __launch_bounds__(32) full_noise_kernel(const void *__restrict__ vis, VisParams P,
                                                         uint32_t n_freq, double f, double N,
                                                         double *s2_out)
@@ -412,16 +392,14 @@ __global__ void __launch_bounds__(32) full_noise_kernel(const void *__restrict__
                     }
                 }
                 const double wi = ok ? D[32 * i] : 0.0, wj = ok ? D[32 * j] : 0.0;
-                const float wif = (float)wi, wjf = (float)wj, wrf = (float)wr, wmf = (float)wm;
-                const float wwf = wif * wjf, re2f = (wrf - wmf) * (wrf + wmf);
                 for (int part = 0; part < 2; part++) {
                     if (part == 1 && i == j) break;
                     const uint32_t comp = part ? NP + p - i - 1 : p;
                     float q = 0.0f;
                     if (ok) {
-                        const float hf = i == j ? wwf : 2.0f * (part ? wwf - re2f : wwf + re2f);
-                        q = __fdividef(f12, hf);
-                        if (s2_out || !(fminf(wif, wjf) > 1e-30f) || !q_beyond_doubt(q, wwf, hf)) {
+                        const bool sure = full_q_f32(f12, (float)wi, (float)wj, (float)wr, (float)wm,
+                                                     i == j, part, q);
+                        if (s2_out || !sure) {
                             const double ww = wi * wj, re2 = wr * wr - wm * wm;
                             const double h = i == j ? N * ww : 2.0 * N * (part ? ww - re2 : ww + re2);
                             const double s2 = 1.0 / h;   // 1 / (C^-1)_kk
