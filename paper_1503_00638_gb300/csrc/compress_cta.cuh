@@ -281,26 +281,39 @@ BSG_D void cta_place(const CodecArgs &a, uint32_t tile, const uint8_t *slot, uin
 }
 
 // Exclusive prefix of a block whose size is published, as lookback_resolve,
-// but at most `looks` looks in vain: LB_UNKNOWN then.  (Looking at 64, 128 or
-// 256 predecessors per step instead of 32 changed nothing: 224-234 us on the
-// 33024 blocks below; sums of groups of 128 blocks by atomics, which thousands
-// of warps read, kept the atomics waiting: 268 to 970 us.)
+// but at most `looks` looks in vain: LB_UNKNOWN then.  With a status word the
+// wait is the last one: when it runs out, or another block's has (the stream is
+// lost then, and one limit is all that the call may wait), it reports
+// BSGPU_ERR_TIMEOUT and publishes what it has added up, so that no successor
+// waits for this block.  (Looking at 64, 128 or 256 predecessors per step
+// instead of 32 changed nothing: 224-234 us on the 33024 blocks below; sums of
+// groups of 128 blocks by atomics, which thousands of warps read, kept the
+// atomics waiting: 268 to 970 us.)
 constexpr uint64_t LB_UNKNOWN = ~0ull;
 
 BSG_D uint64_t lookback_some(uint64_t *state, uint32_t tile, uint64_t agg, uint32_t looks,
-                             uint32_t lane)
+                             int *status, uint32_t lane)
 {
     uint64_t excl = 0;
     uint32_t spins = 0;
+    bool found = true;
     int64_t base = (int64_t)tile - 1;   // blocks base, base - 1, ... are still to be added
     for (bool done = tile == 0; !done;) {
         const int64_t idx = base - (int64_t)lane;
-        const uint64_t v = idx >= 0 ? ld_relaxed_u64(state + idx) : LB_FP;
+        uint64_t v = idx >= 0 ? ld_relaxed_u64(state + idx) : LB_FP;
+#ifdef BSG_TEST_LOOKBACK_STALL
+        if (idx >= 0) v = 0;   // test builds only, as in lookback_resolve
+#endif
         const uint32_t flag = (uint32_t)(v >> 62);
         const uint32_t pm = __ballot_sync(FULL, flag == 2), im = __ballot_sync(FULL, flag == 0);
         const uint32_t first = pm ? (uint32_t)(__ffs(pm) - 1) : 32u;
         if (im & (first >= 32u ? FULL : (1u << first) - 1u)) {
-            if (++spins >= looks) return LB_UNKNOWN;
+            if (++spins >= looks ||
+                (status && spins % 256u == 0 && __any_sync(FULL, *(volatile int *)status != 0))) {
+                if (!status) return LB_UNKNOWN;
+                found = false;
+                break;
+            }
             if (spins > 4096) __nanosleep(100);
             continue;
         }
@@ -313,6 +326,10 @@ BSG_D uint64_t lookback_some(uint64_t *state, uint32_t tile, uint64_t agg, uint3
         base -= 32;
     }
     if (tile && lane == 0) st_relaxed_u64(state + tile, LB_FP | (excl + agg));
+    if (!found) {
+        if (lane == 0) set_status(status, BSGPU_ERR_TIMEOUT);
+        return LB_UNKNOWN;
+    }
     return excl;
 }
 
@@ -435,7 +452,7 @@ BSG_D void compress_cta_body(const CodecArgs &a)
                 },
                 [&] {   // the previous block's place, while this warp has nothing else to do
                     if (ptile != ~0u) {
-                        const uint64_t x = lookback_some(a.tile_state, ptile, 4ull + pcs, 8u, lane);
+                        const uint64_t x = lookback_some(a.tile_state, ptile, 4ull + pcs, 8u, nullptr, lane);
                         if (lane == 0) *excl = x;
                     }
                 });
@@ -450,16 +467,12 @@ BSG_D void compress_cta_body(const CodecArgs &a)
             if (W == 1 || !work || *excl == LB_UNKNOWN) {
                 __syncthreads();   // everyone has seen *excl
                 if (warp == 0) {
-                    uint64_t x = lookback_some(a.tile_state, ptile, 4ull + pcs, 1u << 21, lane);
-                    if (x == LB_UNKNOWN) {
-                        if (lane == 0) set_status(a.status, BSGPU_ERR_TIMEOUT);
-                        x = 0;
-                    }
+                    const uint64_t x = lookback_some(a.tile_state, ptile, 4ull + pcs, 1u << 21, a.status, lane);
                     if (lane == 0) *excl = x;
                 }
                 __syncthreads();
             }
-            cta_place(a, ptile, slot1, pcs, 12 + *excl);
+            if (*excl != LB_UNKNOWN) cta_place(a, ptile, slot1, pcs, 12 + *excl);
         }
         if (!work) break;
         ptile = tile;
@@ -472,8 +485,12 @@ BSG_D void compress_cta_body(const CodecArgs &a)
     // (outside the loop, where it costs the other blocks no registers)
     if (a.tile_begin == 0 && blockIdx.x == 0 && threadIdx.x < 32)
         write_chunk_header(a.out, a.n_elem * ES, a.B * ES, threadIdx.x);
-    if (ptile + 1u == a.nb && threadIdx.x < 32)
-        compress_place_end(a, 12 + *excl + 4 + pcs, threadIdx.x);
+    if (ptile + 1u == a.nb && threadIdx.x < 32) {
+        if (*excl != LB_UNKNOWN)
+            compress_place_end(a, 12 + *excl + 4 + pcs, threadIdx.x);
+        else if (threadIdx.x == 0)
+            *a.out_bytes = 0;   // (the status tells)
+    }
 }
 
 template <int ES, int MODE, uint32_t BC, bool TS>
