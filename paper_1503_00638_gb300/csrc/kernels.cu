@@ -188,18 +188,21 @@ __global__ void __launch_bounds__(256) vis_compensation_kernel(const uint2 *__re
         } else {
             // time-slowest cube: a warp takes one time and its lanes
             // consecutive products, which are neighbours in the input
+            const uint32_t lane = threadIdx.x & 31u;
             for (uint32_t tl = threadIdx.x >> 5; tl < tn; tl += blockDim.x >> 5) {
                 const uint32_t t = t0 + tl;
                 const float *arow = P.autos + (size_t)fr * P.n_in * P.T + t;
                 const uint2 *vrow = vis + (size_t)t * P.FP + (size_t)fr * P.P;
                 CompMax m{0.0f};
-                for (uint32_t pb = p_lo + (threadIdx.x & 31u); pb < p_hi; pb += 4 * 32) {
-                    m.q = __uint_as_float(__reduce_max_sync(__activemask(), __float_as_uint(m.q)));
+                // (the trip count is the warp's, not the lane's: every lane
+                // takes part in the exchange)
+                for (uint32_t pb = p_lo; pb < p_hi; pb += 4 * 32) {
+                    m.q = __uint_as_float(__reduce_max_sync(FULL, __float_as_uint(m.q)));
                     uint2 v[4];
                     uint32_t ijs[4];
 #pragma unroll
                     for (uint32_t k = 0; k < 4; k++) {
-                        const uint32_t p = pb + 32 * k;
+                        const uint32_t p = pb + lane + 32 * k;
                         const bool in = p < p_hi;
                         v[k] = in ? __ldg(vrow + p) : make_uint2(0u, 0u);
                         ijs[k] = in ? __ldg(P.pairs + p) : 0u;
