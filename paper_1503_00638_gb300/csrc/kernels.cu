@@ -45,7 +45,8 @@ uint32_t shuffle_smem_bytes(uint32_t maxb)
 
 // Tables for the rounding: autos[f][i][t] = Re V(f, (i,i), t) and
 // pairs[p] = i | j << 16 for the upper-triangle product order.
-__global__ void vis_tables_kernel(const float *__restrict__ vis, VisParams V, uint32_t n_freq)
+__global__ void vis_tables_kernel(const float *__restrict__ vis, VisParams V, uint32_t n_freq,
+                                  bool zero_cft)
 {
     float *autos = const_cast<float *>(V.autos);
     uint32_t *pairs = const_cast<uint32_t *>(V.pairs);
@@ -64,7 +65,7 @@ __global__ void vis_tables_kernel(const float *__restrict__ vis, VisParams V, ui
         // int32 autos are converted to float32 (round to nearest)
         autos[x] = is_int ? __int2float_rn(reinterpret_cast<const int32_t *>(vis)[at]) : vis[at];
     }
-    if (V.cft)   // the quotients of vis_compensation_kernel start at 0
+    if (zero_cft)   // the quotients of vis_compensation_kernel's slices
         for (uint64_t x = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; x < (uint64_t)n_freq * T;
              x += stride)
             const_cast<float *>(V.cft)[x] = 0.0f;
@@ -165,7 +166,8 @@ __global__ void __launch_bounds__(256) vis_compensation_kernel(const uint2 *__re
                 const uint2 *vrow = vis + (size_t)fr * P.P * P.T + t;
                 CompMax m{0.0f};
                 for (uint32_t pb = p_lo + p0; pb < p_hi; pb += 8 * per) {
-                    m.share(best + tl);
+                    // (before eight more; a single slice knows nothing before its first)
+                    if (pb + 7 * per < p_hi && (slices > 1 || pb != p_lo + p0)) m.share(best + tl);
                     uint2 v[8];
                     uint32_t ijs[8];
 #pragma unroll
@@ -186,17 +188,19 @@ __global__ void __launch_bounds__(256) vis_compensation_kernel(const uint2 *__re
                 m.share(best + tl);
             }
         } else {
-            // time-slowest cube: a warp takes one time and its lanes
-            // consecutive products, which are neighbours in the input
-            const uint32_t lane = threadIdx.x & 31u;
-            for (uint32_t tl = threadIdx.x >> 5; tl < tn; tl += blockDim.x >> 5) {
+            // time-slowest cube: a warp (several, when there are fewer times)
+            // takes one time and its lanes consecutive products, which are
+            // neighbours in the input
+            const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+            const uint32_t wpt = tn < nw ? nw / tn : 1u;   // warps to a time
+            for (uint32_t tl = warp / wpt; tl < tn; tl += nw / wpt) {
                 const uint32_t t = t0 + tl;
                 const float *arow = P.autos + (size_t)fr * P.n_in * P.T + t;
                 const uint2 *vrow = vis + (size_t)t * P.FP + (size_t)fr * P.P;
                 CompMax m{0.0f};
                 // (the trip count is the warp's, not the lane's: every lane
                 // takes part in the exchange)
-                for (uint32_t pb = p_lo; pb < p_hi; pb += 4 * 32) {
+                for (uint32_t pb = p_lo + 4 * 32 * (warp % wpt); pb < p_hi; pb += 4 * 32 * wpt) {
                     m.q = __uint_as_float(__reduce_max_sync(FULL, __float_as_uint(m.q)));
                     uint2 v[4];
                     uint32_t ijs[4];
@@ -226,6 +230,59 @@ __global__ void __launch_bounds__(256) vis_compensation_kernel(const uint2 *__re
                 atomicMax(table + t, best[t]);
         }
         __syncthreads();
+    }
+}
+
+// Few inputs: G lanes (a power of two) take the products of one (freq, time)
+// sample, the autos among them, straight from the cube (neighbouring groups,
+// neighbouring samples: the next time, or in a time-slowest cube the next
+// frequency, whose products follow), with no barrier and no table to read.
+// The CTA per frequency above has too little to do there: 134 MB, whole
+// compensated rounding, 3 inputs x 64 times 282 -> 170 us, in the time-slowest
+// order 751 -> 240; 12 inputs x 5 times 310 -> 173 and 416 -> 229.  (Testing
+// four products together and dividing all four when any may exceed: 122 -> 130
+// us for 12 inputs x 64 times.)
+template <bool INT>
+__global__ void __launch_bounds__(128) vis_compensation_few_kernel(const uint2 *__restrict__ vis,
+                                                                   VisParams P, float *cft,
+                                                                   uint32_t n_freq, uint32_t G,
+                                                                   double f, double N)
+{
+    const uint32_t n = P.n_in, row = P.tslow ? n_freq : P.T, sub = threadIdx.x & (G - 1u);
+    const size_t step = P.tslow ? 1 : P.T;   // from product to product
+    const uint64_t total = (uint64_t)n_freq * P.T;
+    const uint32_t per_cta = blockDim.x / G;
+    for (uint64_t k0 = (uint64_t)blockIdx.x * per_cta; k0 < total; k0 += (uint64_t)gridDim.x * per_cta) {
+        const uint64_t k = k0 + threadIdx.x / G;
+        const uint32_t hi = (uint32_t)(k / row), lo = (uint32_t)(k % row);
+        const uint32_t fr = P.tslow ? lo : hi, t = P.tslow ? hi : lo;
+        const uint2 *v = P.tslow ? vis + (size_t)t * P.FP + (size_t)fr * P.P
+                                 : vis + (size_t)fr * P.P * P.T + t;
+        CompMax m{0.0f};
+        // rows i = sub, sub + G, ... of the products (i, i), (i, i + 1) ..
+        for (uint32_t i = sub; k < total && i + 1 < n; i += G) {
+            const uint32_t pi = i * n - i * (i - 1) / 2;   // product (i, i)
+            const float Ai = comp_sample<INT>(__ldg(v + pi * step)).x;
+            uint32_t pj = pi;   // product (j, j)
+            for (uint32_t j = i + 1; j < n; j += 4) {
+                uint2 x[4], d[4];
+#pragma unroll
+                for (uint32_t u = 0; u < 4; u++) {
+                    const bool in = j + u < n;
+                    pj += in ? n - (j + u - 1) : 0u;
+                    x[u] = in ? __ldg(v + (pi + (j + u - i)) * step) : make_uint2(0u, 0u);
+                    d[u] = in ? __ldg(v + pj * step) : make_uint2(0u, 0u);
+                }
+#pragma unroll
+                for (uint32_t u = 0; u < 4; u++) {
+                    if (j + u >= n) continue;
+                    const float2 z = comp_sample<INT>(x[u]);
+                    m.add(z.x, z.y, Ai, comp_sample<INT>(d[u]).x);
+                }
+            }
+        }
+        for (uint32_t g = 1; g < G; g *= 2) m.q = fmaxf(m.q, __shfl_xor_sync(FULL, m.q, g));
+        if (k < total && sub == 0) cft[(size_t)fr * P.T + t] = compensated_c(__float_as_uint(m.q), f, N);
     }
 }
 
@@ -1326,31 +1383,58 @@ __global__ void __launch_bounds__(32) shuffle_kernel(const __grid_constant__ Cod
 // ---------------------------------------------------------------------------
 // Launchers
 // ---------------------------------------------------------------------------
-cudaError_t launch_vis_compensation(const void *vis, const VisParams &P, uint32_t n_freq,
-                                    double f, double N, cudaStream_t s)
+// Into how many slices the products of a frequency are split (0: a few lanes to
+// each sample).  Up to 12 inputs a sample has no work for a CTA.  From 16 to 32
+// the lanes win when there are samples enough to fill the chip (16 n^2 = 4096
+// to 16384): whole rounding of 134 MB, 24 inputs, 1, 5 and 1000 times: 364,
+// 183 and 146 us in slices, 199, 160 and 121 so; of 8 MB (3500 samples) 31 us
+// in slices and 33 so at 3 times.  64 inputs, 16 times: 112 in slices, 152 so.
+static uint32_t compensation_slices(const VisParams &P, uint32_t n_freq)
 {
+    const uint64_t samples = (uint64_t)n_freq * P.T;
+    if (P.n_in <= 12 || (P.n_in <= 32 && samples >= 16u * P.n_in * P.n_in)) return 0;
     int dev = 0, sms = 148;
     if (cudaGetDevice(&dev) == cudaSuccess)
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     const uint64_t work = (uint64_t)n_freq * ((P.T + 1023) / 1024);
-    // slices of the products: enough CTAs for the eight that are resident per
-    // SM, each thread still with eight samples or more (twice or four times
-    // as many CTAs: 3 and 10 % slower, each starting from less knowledge of
-    // the maximum)
+    // enough CTAs for the eight that are resident per SM, each thread still
+    // with eight samples or more (twice or four times as many CTAs: 3 and
+    // 10 % slower, each starting from less knowledge of the maximum)
     const uint64_t want = ((uint64_t)sms * 8 + work - 1) / work;
     uint64_t most = (uint64_t)P.P * (P.T < 256 ? P.T : 256) / (256 * 8);
     if (most < 1) most = 1;
-    const uint32_t slices = (uint32_t)(want < most ? want : most);
+    return (uint32_t)(want < most ? want : most);
+}
+
+cudaError_t launch_vis_compensation(const void *vis, const VisParams &P, uint32_t n_freq,
+                                    double f, double N, cudaStream_t s)
+{
+    const uint2 *in = reinterpret_cast<const uint2 *>(vis);
     float *cft = const_cast<float *>(P.cft);
     const uint64_t n = (uint64_t)n_freq * P.T;
-    const uint64_t cap = 65536 / slices;
+    const uint32_t slices = compensation_slices(P, n_freq);
+    if (slices == 0) {
+        // as many lanes to a sample as it has rows, until the chip is full; one
+        // step more where they read neighbouring words (time slowest, 134 MB,
+        // 16 inputs x 64 times: 264 us with one lane, 230 with two; time
+        // fastest 111 and 119)
+        const uint64_t full = P.tslow ? 131072 : 65536;
+        uint32_t G = 1;
+        while (2 * G < P.n_in && n * G < full) G *= 2;
+        const uint64_t b = (n * G + 127) / 128;
+        const uint32_t grid = (uint32_t)(b < 65536 ? b : 65536);
+        if (P.is_int)
+            vis_compensation_few_kernel<true><<<grid, 128, 0, s>>>(in, P, cft, n_freq, G, f, N);
+        else
+            vis_compensation_few_kernel<false><<<grid, 128, 0, s>>>(in, P, cft, n_freq, G, f, N);
+        return cudaGetLastError();
+    }
+    const uint64_t work = (uint64_t)n_freq * ((P.T + 1023) / 1024), cap = 65536 / slices;
     const uint32_t grid = (uint32_t)((work < cap ? work : cap) * slices);
     if (P.is_int)
-        vis_compensation_kernel<true><<<grid, 256, 0, s>>>(reinterpret_cast<const uint2 *>(vis), P,
-                                                           cft, n_freq, slices, f, N);
+        vis_compensation_kernel<true><<<grid, 256, 0, s>>>(in, P, cft, n_freq, slices, f, N);
     else
-        vis_compensation_kernel<false><<<grid, 256, 0, s>>>(reinterpret_cast<const uint2 *>(vis), P,
-                                                            cft, n_freq, slices, f, N);
+        vis_compensation_kernel<false><<<grid, 256, 0, s>>>(in, P, cft, n_freq, slices, f, N);
     if (slices > 1) {
         const uint64_t b = (n + 255) / 256;
         vis_compensation_end_kernel<<<(uint32_t)(b < 4096 ? b : 4096), 256, 0, s>>>(cft, n, f, N);
@@ -1390,7 +1474,9 @@ cudaError_t launch_vis_tables(const float *vis, const VisParams &V, uint32_t n_f
     uint32_t blocks = (uint32_t)((work + 255) / 256);
     if (blocks > 4096) blocks = 4096;
     if (blocks == 0) blocks = 1;
-    vis_tables_kernel<<<blocks, 256, 0, s>>>(vis, V, n_freq);
+    // slices that meet in the table start from 0
+    const bool zero = V.cft && compensation_slices(V, n_freq) > 1;
+    vis_tables_kernel<<<blocks, 256, 0, s>>>(vis, V, n_freq, zero);
     return cudaGetLastError();
 }
 
