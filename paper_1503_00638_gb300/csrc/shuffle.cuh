@@ -564,7 +564,7 @@ BSG_D uint64_t transpose8x8(uint64_t x)
     return x;
 }
 
-// With Bb a multiple of 128 a lane takes a group of 128 elements (32 words)
+// With Bb a multiple of 128 (and enough of them, shuf1_wide) a lane takes a group of 128 elements (32 words)
 // through the 32 x 32 transpose instead, in half the instructions: word n of
 // its input holds elements n, n + 32, n + 64 and n + 96 (a 4 x 4 byte
 // transpose of words i, i + 8, i + 16, i + 24), so that word 8 s + r of its
@@ -575,6 +575,11 @@ BSG_D uint64_t transpose8x8(uint64_t x)
 // bits, t as the order of the four words of a bit-row.  256 MiB of bytes,
 // Bitshuffle and back: 205 -> 193 us in 8 KiB blocks (83 % of the copy rate),
 // 236 -> 186 in 4 KiB, 801 -> 514 in 64 KiB (one warp per SM).
+// Blocks of up to 2 KiB keep the other form: a warp has 16 groups there at most,
+// and two passes of 32 elements a lane take as long as one of 128 with half
+// the lanes idle (64 MiB, Bitshuffle: 2 KiB 45 and 49 us, 1 KiB 61 and 89,
+// 512 bytes 114 and 169; 4 KiB 36 and 28).
+BSG_HD bool shuf1_wide(uint32_t Bb) { return Bb % 128u == 0 && Bb > 2048u; }
 BSG_HD uint32_t shuf1_flip(uint32_t g) { return (g >> 2) & 1u; }
 BSG_HD uint32_t shuf1_turn(uint32_t g) { return ((g & 3u) + (g >> 3)) & 3u; }
 
@@ -661,7 +666,7 @@ BSG_D void unshuf1_store_group(uint8_t *grp, uint32_t g, uint32_t (&v)[32])
 BSG_D void shuffle1_fast(const uint8_t *src, uint8_t *dst, uint32_t Bb, uint32_t lane)
 {
     const uint32_t Q = Bb / 32;  // groups of 32 elements; also words per bit-row
-    if (Bb % 128u == 0) {
+    if (shuf1_wide(Bb)) {
         for (uint32_t g = lane; g < Bb / 128u; g += 32) {
             uint32_t v[32];
             shuf1_read_group(src + 128u * g, g, v);
@@ -693,7 +698,7 @@ BSG_D void unshuffle1_fast(const uint8_t *src, uint8_t *dst, uint32_t Bb, uint32
                             uint32_t step = 32)
 {
     const uint32_t Q = Bb / 32;
-    if (Bb % 128u == 0) {
+    if (shuf1_wide(Bb)) {
         for (uint32_t g = lane; g < Bb / 128u; g += step) {
             uint32_t v[32];
             unshuf1_get_rows(src, Q, g, v);
