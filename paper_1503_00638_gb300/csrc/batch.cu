@@ -312,7 +312,7 @@ BSG_D bool batch_decode(const BatchArgs &b, uint32_t c, uint32_t tile, const Dec
         if (cur.eidx != ~0u) comp[cur.eidx] = cur.ebyte;
         __syncwarp();
         good = get_be32(comp + cur.delta) == cur.clen &&
-               lz4_decode_warp(dec, cur.off + cur.delta + 4, cur.clen, dec, Bb * ch.es) == 0;
+               lz4_decode_warp<true>(dec, cur.off + cur.delta + 4, cur.clen, dec, Bb * ch.es) == 0;
     }
     if (!good && lane == 0) set_status(b.status + c, BSGPU_ERR_CORRUPT);
     return good;

@@ -774,8 +774,10 @@ __global__ void __launch_bounds__(32, 20) decompress_inplace_kernel(const __grid
         if (good) {
             if (cur.eidx != ~0u) comp[cur.eidx] = cur.ebyte;
             __syncwarp();
+            // (both forms are the same; each is the one whose registers fit)
             good = get_be32(comp + cur.delta) == cur.clen &&
-                   lz4_decode_warp(buf, cur.off + cur.delta + 4, cur.clen, buf, S) == 0;
+                   (ES == 8 ? lz4_decode_warp<true>(comp, cur.delta + 4, cur.clen, buf, S)
+                            : lz4_decode_warp<true>(buf, cur.off + cur.delta + 4, cur.clen, buf, S)) == 0;
         }
         if (!good && lane == 0) set_status(a.status, BSGPU_ERR_CORRUPT);
         __syncwarp();
@@ -874,7 +876,7 @@ __global__ void __launch_bounds__(32, 20) decompress_inplace_any_kernel(const __
             if (cur.eidx != ~0u) comp[cur.eidx] = cur.ebyte;
             __syncwarp();
             good = get_be32(comp + cur.delta) == cur.clen &&
-                   lz4_decode_warp(buf, cur.off + cur.delta + 4, cur.clen, buf, S) == 0;
+                   lz4_decode_warp<true>(buf, cur.off + cur.delta + 4, cur.clen, buf, S) == 0;
         }
         if (!good && lane == 0) set_status(a.status, BSGPU_ERR_CORRUPT);
         __syncwarp();

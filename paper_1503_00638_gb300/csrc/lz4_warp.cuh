@@ -981,12 +981,13 @@ BSG_D void lz4_match_copy(uint8_t *dst, uint32_t op, uint32_t off, uint32_t ML, 
 
 // Strict decode of the clen bytes src[ip0 ..] into exactly S bytes of dst
 // (src and dst word-aligned shared buffers; src readable 8 bytes past the
-// end; src == dst when decoding in place).  Returns 0, or a nonzero code for:
+// end; IN_PLACE: src lies in dst's buffer, src - dst bytes on).  Returns 0, or a nonzero code for:
 // input ending early (1), a literal run overrunning the output (2), a bad
 // offset or match length, or a match breaking the end-of-block rules or
 // running into unread input (3), a final length other than S (6).
 // The token and the offset are each read together with the byte after them
 // (one funnel-shifted word), so a length of 15..269 costs no extra read.
+template <bool IN_PLACE = false>
 BSG_D int lz4_decode_warp(const uint8_t *src, uint32_t ip0, uint32_t clen, uint8_t *dst,
                           uint32_t S)
 {
@@ -1031,9 +1032,8 @@ BSG_D int lz4_decode_warp(const uint8_t *src, uint32_t ip0, uint32_t clen, uint8
         }
         ML += LZ4_MINMATCH;
         // (ML is below 2^31: at most 255 per stream byte)
-        // In place the match must not reach the unread input either: by
-        // decompress_inplace_kernel's margin only a corrupt block's would.
-        const uint32_t most = S - LZ4_LASTLITERALS, room = src == dst && ip < most ? ip : most;
+        const uint32_t most = S - LZ4_LASTLITERALS, read = ip + (uint32_t)(src - dst);
+        const uint32_t room = IN_PLACE && read < most ? read : most;
         if ((off == 0) | (off > op) | (op + ML > room) | (op + LZ4_MFLIMIT > S))
             return 3;
         __syncwarp();

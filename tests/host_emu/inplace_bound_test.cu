@@ -53,7 +53,7 @@ int main(int argc, char **argv)
                 bool ok = false;
                 run_cta(32 * warps, [&] {
                     const bool r = warps == 2 ? cta_lz4_decode(D, ip0, clen, D, S, ring, threadIdx.x)
-                                              : lz4_decode_warp(D, ip0, clen, D, S) == 0;
+                                              : lz4_decode_warp<true>(D + off, ph + 4, clen, D, S) == 0;
                     if (threadIdx.x == 0) ok = r;
                 });
                 const bool whole = memcmp(D + ip0 + read, img.data() + read, clen - read) == 0;
