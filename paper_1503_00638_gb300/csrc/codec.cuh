@@ -702,7 +702,14 @@ struct NoRound {
 // safety (image start - (S - clen) >= 72).
 constexpr uint32_t INPLACE_BUF = 8352;
 
-static_assert(INPLACE_BUF >= 4 + lz4b(8192) + 48 && INPLACE_BUF >= 8192 + 2 * 8192 / 255 + 49,
+// The same for blocks of any size up to maxb.
+__host__ __device__ constexpr uint32_t inplace_any_buf(uint32_t maxb)
+{
+    return maxb <= 8192 ? INPLACE_BUF : r16(maxb + 2u * maxb / 255u + 160u);
+}
+static_assert(inplace_any_buf(16384) >= 4 + lz4b(16384) + 48 &&
+                  inplace_any_buf(16384) >= 16384 + 2 * 16384 / 255 + 49 &&
+                  INPLACE_BUF >= 4 + lz4b(8192) + 48 && INPLACE_BUF >= 8192 + 2 * 8192 / 255 + 49,
               "in-place buffer");
 static_assert(INPLACE_BUF >= 8192 + 119, "in-place buffer: margin below the LZ4 bound");
 

@@ -44,9 +44,11 @@ BSG_D void dec_check_header(const CodecArgs &a, uint32_t lane)
 // 16, 32 and 64 KiB: 164, 258 and 424 us with one warp per block, 155, 212 and
 // 334 us with two.  Blocks of at most 8 KiB keep one warp (the in-place kernel
 // of kernels.cu): there 20 parsing warps per SM are issue-bound, and two warps
-// a block, 16 blocks per SM, took 1.25 to 1.6 times as long.
+// a block, 16 blocks per SM, took 1.25 to 1.6 times as long.  8-byte
+// elements keep one warp up to 16 KiB too, and have 96 registers above (with 80
+// their un-transpose spilled: 67 MB in 32 KiB blocks 69 -> 65 us).
 template <int ES>
-__global__ void __launch_bounds__(64, 12) decompress_cta_kernel(const __grid_constant__ CodecArgs a)
+__global__ void __launch_bounds__(64, ES == 8 ? 10 : 12) decompress_cta_kernel(const __grid_constant__ CodecArgs a)
 {
     extern __shared__ __align__(128) uint8_t sm[];
     const uint32_t BUF = dec_cta_buf(a.B * ES);

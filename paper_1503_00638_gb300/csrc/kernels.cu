@@ -826,17 +826,22 @@ __global__ void __launch_bounds__(32, 20) decompress_inplace_kernel(const __grid
     __syncwarp();
 }
 
-// In-place decoding for 1-byte elements in blocks of at most 8 KiB: one buffer
-// per warp with the block's compressed image near its end and the bit-rows
-// decoded from its start, un-transposed from there straight into the output,
-// which is 16-byte aligned for every block (the caller checks B * es).  The
-// margin argument above holds for any S: the LZ4 bytes must start at least 2 +
-// 2 S / 255 bytes after S - clen, and dec_issue puts them at least E - clen -
-// 47 bytes in (E the buffer size), so E >= S + 2 S / 255 + 49 suffices.
-// (Blocks over 8 KiB: decompress_cta.cuh.)
-__global__ void __launch_bounds__(32, 20) decompress_inplace_any_kernel(const __grid_constant__ CodecArgs a)
+// In-place decoding for 1-byte elements in blocks of at most 8 KiB and 8-byte
+// elements in blocks of up to 16 KiB: one buffer per warp with the block's
+// compressed image near its end and the bit-rows decoded from its start,
+// un-transposed from there straight into the output, which is 16-byte aligned
+// for every block (the caller checks B * es).  The margin argument above holds
+// for any S: the LZ4 bytes must start at least 2 + 2 S / 255 bytes after S -
+// clen, and dec_issue puts them at least E - clen - 47 bytes in (E the buffer
+// size), so E >= S + 2 S / 255 + 49 suffices.  (Other blocks over 8 KiB: the
+// two warps of decompress_cta.cuh.  8-byte walks have few sequences, which
+// leaves the second warp idle, and two warps' registers hold fewer blocks: 67
+// MB in blocks of 12 and 16 KiB 51 and 50 us here, 62 and 56 with two warps; in
+// 32 KiB 72 and 65.)
+template <uint32_t MAXB>
+__global__ void __launch_bounds__(32, MAXB <= 8192 ? 20 : 12) decompress_inplace_any_kernel(const __grid_constant__ CodecArgs a)
 {
-    constexpr uint32_t BUF = INPLACE_BUF;
+    constexpr uint32_t BUF = inplace_any_buf(MAXB);
     extern __shared__ __align__(128) uint8_t sm[];
     uint8_t *buf = sm;
     uint64_t *bar = reinterpret_cast<uint64_t *>(sm + BUF);
@@ -897,7 +902,7 @@ __global__ void __launch_bounds__(32, 20) decompress_inplace_any_kernel(const __
     }
 }
 
-uint32_t decompress_inplace_any_smem_bytes() { return INPLACE_BUF + 16; }
+uint32_t decompress_inplace_any_smem_bytes(uint32_t maxb) { return inplace_any_buf(maxb) + 16; }
 
 uint32_t decompress_inplace_blocks_per_sm(uint32_t es)
 {
@@ -1684,9 +1689,11 @@ cudaError_t launch_decompress(const CodecArgs &a, uint32_t maxb, uint32_t grid, 
     return launch_warp_kernel(decompress_kernel<65536, 0>, smem, grid, s, a);
 }
 
-cudaError_t launch_decompress_inplace_any(const CodecArgs &a, uint32_t grid, cudaStream_t s)
+cudaError_t launch_decompress_inplace_any(const CodecArgs &a, uint32_t maxb, uint32_t grid, cudaStream_t s)
 {
-    return launch_warp_kernel(decompress_inplace_any_kernel, decompress_inplace_any_smem_bytes(), grid, s, a);
+    const uint32_t smem = decompress_inplace_any_smem_bytes(maxb);
+    return maxb <= 8192 ? launch_warp_kernel(decompress_inplace_any_kernel<8192>, smem, grid, s, a)
+                        : launch_warp_kernel(decompress_inplace_any_kernel<16384>, smem, grid, s, a);
 }
 
 cudaError_t launch_chain_walk(const CodecArgs &a, uint64_t *offsets, void *seg_ws,

@@ -81,7 +81,7 @@ uint32_t decompress_smem_bytes(uint32_t maxb);
 // resident CTAs per SM of the one-buffer (in-place) decompress kernel
 uint32_t decompress_inplace_blocks_per_sm(uint32_t es);
 // shared memory of the in-place decompress kernel for other shapes
-uint32_t decompress_inplace_any_smem_bytes();
+uint32_t decompress_inplace_any_smem_bytes(uint32_t maxb);
 uint32_t shuffle_smem_bytes(uint32_t maxb);
 
 // Launchers (return cudaGetLastError()).  `grid` warps of 32 threads.
@@ -130,10 +130,11 @@ cudaError_t launch_compress_cta_group_x(const CodecArgs &a, uint32_t max_ctas, c
 cudaError_t launch_compress_cta_sample(const CodecArgs &a, uint32_t max_ctas, cudaStream_t s);
 cudaError_t launch_compress_small(const CodecArgs &a, cudaStream_t s);
 cudaError_t launch_decompress(const CodecArgs &a, uint32_t maxb, uint32_t grid, cudaStream_t s);
-// In-place decoding of 1-byte elements in blocks of at most 8 KiB, the output
-// 16-byte aligned for every block ((a.B * a.es) % 16 == 0, a.out aligned).
-cudaError_t launch_decompress_inplace_any(const CodecArgs &a, uint32_t grid, cudaStream_t s);
-// Decompressor of blocks over 8 KiB, a CTA of two warps per block
+// In-place decoding of 1-byte elements in blocks of at most 8 KiB and 8-byte
+// elements in blocks of up to 16 KiB (maxb: the size class), the output 16-byte
+// aligned for every block ((a.B * a.es) % 16 == 0, a.out aligned).
+cudaError_t launch_decompress_inplace_any(const CodecArgs &a, uint32_t maxb, uint32_t grid, cudaStream_t s);
+// Decompressor of other blocks over 8 KiB, a CTA of two warps per block
 // (decompress_cta.cu), the output 16-byte aligned for every block ((a.B * a.es) % 16 == 0, a.out aligned).
 cudaError_t launch_decompress_cta(const CodecArgs &a, cudaStream_t s);
 // Block index of a stream without one (seg_ws: SEG_WS_BYTES of workspace for
