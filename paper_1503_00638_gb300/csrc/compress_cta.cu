@@ -8,7 +8,7 @@ namespace bsg {
 
 uint32_t compress_cta_max(uint32_t S, uint32_t sms)
 {
-    // (the larger of the two levels)
+    // (the larger of the two levels, with the usual tables)
     const uint32_t s0 = cta_plan<0>(S).smem, s1 = cta_plan<1>(S).smem, W = cta_plan<0>(S).W;
     uint32_t p0 = (228u * 1024u) / (s0 + 1024u), p1 = (228u * 1024u) / (s1 + 1024u);
     if (p0 > 32u / W) p0 = 32u / W;
@@ -31,7 +31,7 @@ cudaError_t launch_compress_cta(const CodecArgs &a, uint32_t max_ctas, cudaStrea
     switch (a.es) {
     case 1: return launch_compress_cta1(a, max_ctas, s);
     case 2: return launch_compress_cta2(a, max_ctas, s);
-    case 4: return launch_cta_stream<0, 4, CTA_PLAIN, 2048, 1024, 4096, 8192>(a, max_ctas, s);
+    case 4: return launch_cta_stream<0, 4, CTA_PLAIN, 2048, 1024, 512, 4096, 8192>(a, max_ctas, s);
     default: return launch_compress_cta8(a, max_ctas, s);
     }
 }

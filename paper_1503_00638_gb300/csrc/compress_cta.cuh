@@ -45,11 +45,27 @@ __host__ __device__ constexpr uint32_t cta_warps_of(uint32_t S)
     return LEVEL >= 1 ? (S + 8191u) / 8192u : cta_warps(S);
 }
 
+// Nodes for the parse graph of a kernel with a fixed block size of S bytes (0:
+// the usual number, 64 a warp).  Cubes have few, other data up to one to 28
+// bytes.  64 MiB of which one byte in 33 is not zero has 72 nodes to 2 KiB and
+// 290 to 8 KiB on average: 450 us in blocks of 2 KiB and 400 in 8 KiB with 64 a
+// warp (the one-warp encoder with its 128: 282 and 381), 190 and 260 so.  At 4
+// KiB, where 64 are no slower than that encoder was (242 and 371 us), more
+// would cost other data shared memory and L1 (walks 79 -> 81 us; int32 cube in
+// the instrument's order 252 -> 260).
+template <int MODE>
+__host__ __device__ constexpr uint32_t cta_fixed_cap(uint32_t S)
+{
+    if (MODE != CTA_PLAIN) return 0;
+    return S <= 2048u ? 96u : S > 4096u && S <= 8192u ? 320u : 0u;
+}
+
+// (cap: nodes of level 0's tables, 0 for the usual number)
 template <int LEVEL>
-__host__ __device__ constexpr CtaPlan cta_plan(uint32_t S)
+__host__ __device__ constexpr CtaPlan cta_plan(uint32_t S, uint32_t cap = 0)
 {
     const uint32_t W = cta_warps_of<LEVEL>(S), tmp = r16(S + 16u);
-    return CtaPlan{W, tmp, tmp + r16(cta_scratch_bytes<LEVEL>(W, cta_hbits(S))) + 16u,
+    return CtaPlan{W, tmp, tmp + r16(cta_scratch_bytes<LEVEL>(W, cta_hbits(S), cap)) + 16u,
                    r16(4u + lz4b(S) + 32u)};
 }
 
@@ -348,8 +364,8 @@ BSG_D uint64_t lookback_some(uint64_t *state, uint32_t tile, uint64_t agg, uint3
 // 32 KiB blocks, which took a kernel of two buffers per warp: 0.88 -> 0.18 ms.
 //
 // BC: the block size in elements when it is one of the usual ones (4 and 8
-// KiB, 16 and 32 KiB of 4- and 8-byte elements; full blocks only), else 0 for
-// any size and for a shortened last block.  With the size known the strides of
+// KiB; but for cubes 2 KiB and, of 4- and 8-byte elements, 16 and 32; full blocks
+// only), else 0 for any size and for a shortened last block.  With the size known the strides of
 // the bit-rows, the loops over the warps and the tables' places are constants
 // (int32 cube, time slowest, as 8-byte samples in 4 KiB blocks, 127 MB: 279 ->
 // 253 us; 268 MB of float64 in 32 KiB blocks: 206 -> 182 us).  TS: a
@@ -359,10 +375,11 @@ BSG_D void compress_cta_body(const CodecArgs &a)
 {
     extern __shared__ __align__(128) uint8_t sm[];
     const uint32_t W = BC ? cta_warps(BC * ES) : blockDim.x >> 5;
-    const CtaPlan plan = cta_plan<LEVEL>((BC ? BC : a.B) * ES);
+    constexpr uint32_t CAP = BC ? cta_fixed_cap<MODE>(BC * ES) : 0u;
+    const CtaPlan plan = cta_plan<LEVEL>((BC ? BC : a.B) * ES, CAP);
     const uint32_t hbits = cta_hbits((BC ? BC : a.B) * ES);
     uint8_t *buf = sm;
-    const CtaScratch c = cta_scratch<LEVEL>(sm + plan.tmp, W, hbits);
+    const CtaScratch c = cta_scratch<LEVEL>(sm + plan.tmp, W, hbits, CAP);
     uint64_t *bar = reinterpret_cast<uint64_t *>(sm + plan.smem - 16u);
     uint32_t *next = c.ex + EX_CTL + 2;            // the next tile
     uint64_t *excl = reinterpret_cast<uint64_t *>(c.ex + EX_CTL + 4);
@@ -516,7 +533,7 @@ __global__ void __maxnreg__(CTA_L1_REGS)
 template <int LEVEL, int ES, int MODE, uint32_t BC, bool TS = false>
 cudaError_t launch_cta(const CodecArgs &a, uint32_t max_ctas, cudaStream_t s)
 {
-    const CtaPlan plan = cta_plan<LEVEL>(a.B * ES);
+    const CtaPlan plan = cta_plan<LEVEL>(a.B * ES, BC ? cta_fixed_cap<MODE>(BC * ES) : 0u);
     auto kernel = compress_cta_kernel<ES, MODE, BC, TS>;
     if constexpr (LEVEL >= 1) kernel = compress_cta_l1_kernel<ES, MODE, TS>;
     if (plan.smem > 48 * 1024) {

@@ -7,7 +7,7 @@ namespace bsg {
 
 cudaError_t launch_compress_cta8(const CodecArgs &a, uint32_t max_ctas, cudaStream_t s)
 {
-    return launch_cta_stream<0, 8, CTA_PLAIN, 1024, 512, 2048, 4096>(a, max_ctas, s);
+    return launch_cta_stream<0, 8, CTA_PLAIN, 1024, 512, 256, 2048, 4096>(a, max_ctas, s);
 }
 
 cudaError_t launch_compress_cta_vis8(const CodecArgs &a, uint32_t max_ctas, cudaStream_t s)

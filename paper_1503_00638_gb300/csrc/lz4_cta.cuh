@@ -52,13 +52,20 @@ BSG_D uint32_t fresh_tid()
 #endif
 }
 
-// Nodes of the parse graph that the tables hold; a block with more walks
-// from candidate to match end (the same bytes).  The CHIME-shaped data has
-// 32 nodes per 8 KiB block on average, 80 at most.
-__host__ __device__ constexpr uint32_t cta_node_cap(uint32_t W) { return 64u * W; }
-
 // Warps for a block of S bytes: one thread per 128 bytes.
 __host__ __device__ constexpr uint32_t cta_warps(uint32_t S) { return (S + 4095u) / 4096u; }
+
+// Nodes of the parse graph that the tables hold for W warps' blocks unless the
+// caller gives more room; a block with more walks from candidate to match end
+// (the same bytes).  The CHIME-shaped data has 32 nodes per 8 KiB block on
+// average, 80 at most.
+__host__ __device__ constexpr uint32_t cta_node_cap(uint32_t W) { return 64u * W; }
+// Words of the bitmaps and, over them, of the four jump tables.
+__host__ __device__ constexpr uint32_t cta_bitmap_words(uint32_t W, uint32_t cap)
+{
+    const uint32_t maps = 2u * (32u * W + 1u) + 5u * 32u * W, jumps = 2u * cap;
+    return maps > jumps ? maps : jumps;
+}
 
 constexpr uint32_t CTA_MAX_WARPS = 16;   // 64 KiB blocks
 constexpr uint32_t CTA_NONE = 0xffffu;
@@ -77,23 +84,26 @@ struct CtaScratch {
     uint32_t *ex;     // exchange words between the warps (EX_*)
     uint16_t *table;  // level 1: the hash table (2^hbits entries), the rest but
                       // desc and ex unused
-    uint16_t *jmp;    // jump tables: over E, cer and ceu, dead by then
+    uint16_t *jmp;    // jump tables: over E to pre, dead by then
+    uint32_t cap;     // nodes the tables hold, 0 for cta_node_cap(W)
 };
 enum : uint32_t { EX_NZ = 0, EX_CNT = 16, EX_SCAN = 32, EX_LIT = 48, EX_CTL = 64, EX_WORDS = 72 };
 
 // Hash bits of level 1 for blocks of S bytes.
 __host__ __device__ constexpr uint32_t cta_hbits(uint32_t S) { return S <= 8192u ? 11u : S <= 16384u ? 12u : 13u; }
 
+// (level 0: with tables of `cap` nodes, 0 for cta_node_cap(W))
 template <int LEVEL>
-__host__ __device__ constexpr uint32_t cta_scratch_bytes(uint32_t W, uint32_t hbits = 0)
+__host__ __device__ constexpr uint32_t cta_scratch_bytes(uint32_t W, uint32_t hbits = 0, uint32_t cap = 0)
 {
     return LEVEL >= 1 ? (2u << hbits) + 4u * (2u * (32u * W + 1u) + EX_WORDS)
-                      : 4u * (2u * (32u * W + 1u) + 5u * 32u * W + 2u * cta_node_cap(W) +
+                      : 4u * ((cap ? cta_bitmap_words(W, cap) + 2u * cap
+                                   : 2u * (32u * W + 1u) + 5u * 32u * W + 2u * cta_node_cap(W)) +
                               2u * (32u * W + 1u) + EX_WORDS);
 }
 
 template <int LEVEL>
-BSG_D CtaScratch cta_scratch(uint8_t *base, uint32_t W, uint32_t hbits = 0)
+BSG_D CtaScratch cta_scratch(uint8_t *base, uint32_t W, uint32_t hbits = 0, uint32_t cap = 0)
 {
     CtaScratch c{};
     uint32_t *p = reinterpret_cast<uint32_t *>(base);   // 16-byte aligned
@@ -101,6 +111,8 @@ BSG_D CtaScratch cta_scratch(uint8_t *base, uint32_t W, uint32_t hbits = 0)
         c.table = reinterpret_cast<uint16_t *>(p);
         p += (2u << hbits) / 4u;
     } else {
+        uint32_t *const end = p + (cap ? cta_bitmap_words(W, cap) : 0u);
+        c.cap = cap;
         c.E = reinterpret_cast<uint2 *>(p);
         c.jmp = reinterpret_cast<uint16_t *>(p);
         p += 2u * (32u * W + 1u);
@@ -110,14 +122,16 @@ BSG_D CtaScratch cta_scratch(uint8_t *base, uint32_t W, uint32_t hbits = 0)
         c.row = p + 96u * W;
         c.pre = p + 128u * W;
         p += 160u * W;
+        if (cap) p = end;
         c.node = reinterpret_cast<uint2 *>(p);
-        p += 2u * cta_node_cap(W);
+        p += 2u * (cap ? cap : cta_node_cap(W));
     }
     c.desc = reinterpret_cast<uint2 *>(p);
     p += 2u * (32u * W + 1u);
     c.ex = p;
     return c;
 }
+
 // the four jump tables fit the space of the bitmaps they replace
 static_assert(4u * cta_node_cap(1) * 2u <= 4u * (2u * 33u + 64u), "jump tables");
 
@@ -183,7 +197,7 @@ BSG_D uint32_t cta_lz4_encode(const uint8_t *src, uint32_t S, uint32_t rowlen, u
     const uint32_t *s32 = reinterpret_cast<const uint32_t *>(src);
     const uint32_t NB = (S / 4u + 31u) / 32u;
     const uint32_t R = (rowlen & 3u) ? 0u : rowlen / 4u;
-    const uint32_t cap_nodes = cta_node_cap(W);
+    const uint32_t cap_nodes = c.cap ? c.cap : cta_node_cap(W);
 
     const bool some = LEVEL >= 1 || (S >= LZ4_MFLIMIT + 1u && S >= LZ4_LASTLITERALS + LZ4_L0_MINMATCH);
     const uint32_t wlim = some ? (S - LZ4_LASTLITERALS - LZ4_L0_MINMATCH) / 4u : 0u;
