@@ -455,7 +455,7 @@ BSG_D void compress_cta_body(const CodecArgs &a)
                     }
                 }
             } else {
-                cta_eq_bitmaps(s32, S / 4u, R, c, W);
+                cta_eq_bitmaps<BC && ES <= 2 ? 8 : 1>(s32, S / 4u, R, c, W);
             }
             if (LEVEL == 0) __syncthreads();
             cs = cta_lz4_encode<LEVEL>(

@@ -25,7 +25,7 @@ int main(int argc, char **argv)
         uint32_t cs = 0, want = 0;
         run_cta(32 * W, [&] {
             const CtaScratch c = cta_scratch<0>(scr, W, 0, cap);
-            cta_eq_bitmaps(w, NW, rowlen / 4, c, W);
+            cta_eq_bitmaps<1>(w, NW, rowlen / 4, c, W);
             __syncthreads();
             const uint32_t o = cta_lz4_encode<0>(buf, S, rowlen, out + 4, c, W, 0, [](uint32_t) {}, [] {});
             if (threadIdx.x == 0) cs = o;
