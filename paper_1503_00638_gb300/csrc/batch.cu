@@ -485,8 +485,7 @@ template <typename K>
 uint32_t occupancy(K kernel, uint32_t smem, uint32_t warps)
 {
     int n = 0;
-    if (smem > 48 * 1024)
-        cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    allow_smem(kernel, smem);
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kernel, (int)(32 * warps), smem) !=
             cudaSuccess || n < 1)
         n = 1;
@@ -497,11 +496,8 @@ template <typename K>
 cudaError_t launch_batch(K kernel, uint32_t smem, uint32_t grid, uint32_t warps, cudaStream_t s,
                          const BatchArgs &b)
 {
-    if (smem > 48 * 1024) {
-        cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             (int)smem);
-        if (e != cudaSuccess) return e;
-    }
+    const cudaError_t e = allow_smem(kernel, smem);
+    if (e != cudaSuccess) return e;
     kernel<<<grid, 32 * warps, smem, s>>>(b);
     return cudaGetLastError();
 }
@@ -682,10 +678,7 @@ int bsgpu_decompress_batch_ex(const void *d_table, uint32_t n_chunks, uint64_t n
         b.offsets = const_cast<uint64_t *>(d_block_offsets);
     } else {
         b.offsets = reinterpret_cast<uint64_t *>((uint8_t *)ws + w.offsets);
-        if (cudaFuncSetAttribute(chain_walk_batch_kernel,
-                                 cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)WALK_SMEM) != cudaSuccess)
-            return BSGPU_ERR_CUDA;
+        if (allow_smem(chain_walk_batch_kernel, WALK_SMEM) != cudaSuccess) return BSGPU_ERR_CUDA;
         const uint32_t g = (uint32_t)(n_chunks < (uint32_t)sm_count() ? n_chunks : sm_count());
         chain_walk_batch_kernel<<<g, 32, WALK_SMEM, s>>>(b);
         if (cudaGetLastError() != cudaSuccess) return BSGPU_ERR_CUDA;

@@ -965,15 +965,26 @@ BSG_D bool seg_plausible(const uint8_t *in, uint64_t p, uint64_t end, uint32_t m
     return true;
 }
 
+// Let a kernel be launched with `smem` bytes of dynamic shared memory.  Its limit
+// is raised to all that a CTA can have, never to one call's size: kernels are
+// shared by calls of several sizes, and a thread with a smaller one would
+// refuse another thread's launch between its two steps.
+constexpr int SMEM_LIMIT = 227 * 1024;
+
+template <typename K>
+inline cudaError_t allow_smem(K kernel, uint32_t smem)
+{
+    return smem <= 48u * 1024u ? cudaSuccess
+                               : cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                      SMEM_LIMIT);
+}
+
 template <typename K>
 inline cudaError_t launch_warp_kernel(K kernel, uint32_t smem, uint32_t grid, cudaStream_t s,
                                       const CodecArgs &a)
 {
-    if (smem > 48 * 1024) {
-        cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             (int)smem);
-        if (e != cudaSuccess) return e;
-    }
+    const cudaError_t e = allow_smem(kernel, smem);
+    if (e != cudaSuccess) return e;
     kernel<<<grid, 32, smem, s>>>(a);
     return cudaGetLastError();
 }

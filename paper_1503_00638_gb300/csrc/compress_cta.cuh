@@ -536,11 +536,8 @@ cudaError_t launch_cta(const CodecArgs &a, uint32_t max_ctas, cudaStream_t s)
     const CtaPlan plan = cta_plan<LEVEL>(a.B * ES, BC ? cta_fixed_cap<MODE>(BC * ES) : 0u);
     auto kernel = compress_cta_kernel<ES, MODE, BC, TS>;
     if constexpr (LEVEL >= 1) kernel = compress_cta_l1_kernel<ES, MODE, TS>;
-    if (plan.smem > 48 * 1024) {
-        const cudaError_t e = cudaFuncSetAttribute(
-            kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)plan.smem);
-        if (e != cudaSuccess) return e;
-    }
+    const cudaError_t e = allow_smem(kernel, plan.smem);
+    if (e != cudaSuccess) return e;
     int dev = 0, sms = 148, per = 1;
     if (cudaGetDevice(&dev) == cudaSuccess)
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);

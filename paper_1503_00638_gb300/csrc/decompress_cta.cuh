@@ -116,11 +116,8 @@ cudaError_t launch_decompress_cta_es(const CodecArgs &a, cudaStream_t s)
 {
     auto kernel = decompress_cta_kernel<ES>;
     const uint32_t smem = dec_cta_smem(a.B * ES);
-    if (smem > 48 * 1024) {
-        const cudaError_t e = cudaFuncSetAttribute(
-            kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-    }
+    const cudaError_t e = allow_smem(kernel, smem);
+    if (e != cudaSuccess) return e;
     int dev = 0, sms = 148, per = 1;
     if (cudaGetDevice(&dev) == cudaSuccess)
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);

@@ -1458,8 +1458,7 @@ cudaError_t launch_full_noise(const void *vis, const VisParams &P, uint32_t n_fr
                               double N, double *s2, cudaStream_t s)
 {
     const uint32_t smem = full_noise_smem_bytes(P.n_in);
-    cudaError_t e = cudaFuncSetAttribute(full_noise_kernel,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    const cudaError_t e = allow_smem(full_noise_kernel, smem);
     if (e != cudaSuccess) return e;
     int dev = 0, sms = 148, per = 1;
     if (cudaGetDevice(&dev) == cudaSuccess)
@@ -1590,11 +1589,8 @@ template <typename K>
 cudaError_t launch_tiles(K kernel, uint32_t smem, uint32_t grid, cudaStream_t s, const CodecArgs &a,
                          uint32_t nfull)
 {
-    if (smem > 48 * 1024) {
-        cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             (int)smem);
-        if (e != cudaSuccess) return e;
-    }
+    const cudaError_t e = allow_smem(kernel, smem);
+    if (e != cudaSuccess) return e;
     kernel<<<grid, 32, smem, s>>>(a, nfull);
     return cudaGetLastError();
 }
@@ -1699,8 +1695,7 @@ cudaError_t launch_decompress_inplace_any(const CodecArgs &a, uint32_t maxb, uin
 cudaError_t launch_chain_walk(const CodecArgs &a, uint64_t *offsets, void *seg_ws,
                               cudaStream_t s)
 {
-    cudaError_t e = cudaFuncSetAttribute(chain_walk_kernel,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)WALK_SMEM);
+    cudaError_t e = allow_smem(chain_walk_kernel, WALK_SMEM);
     if (e != cudaSuccess) return e;
     uint32_t *verified = nullptr;
     if (seg_ws) {

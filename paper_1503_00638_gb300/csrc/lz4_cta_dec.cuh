@@ -152,7 +152,7 @@ BSG_D bool cta_lz4_decode(const uint8_t *src, uint32_t ip0, uint32_t clen, uint8
                 // (ML is below 2^31: at most 255 per stream byte)
                 // In place the match must not reach what the parser has still to
                 // read either: by that margin only a corrupt block's would.
-                const uint32_t most = S - LZ4_LASTLITERALS, room = src == dst && ip < most ? ip : most;
+                const uint32_t last = S - LZ4_LASTLITERALS, room = src == dst && ip < last ? ip : last;
                 if ((off == 0) | (off > op) | (op + ML > room) | (op + LZ4_MFLIMIT > S)) break;
                 if (lane == 0) seq[half + n] = make_uint2(op | (off << 16), ML);
                 op += ML;

@@ -16,3 +16,15 @@ def test_warp_collectives_name_lanes_known_beforehand(path):
     the next instruction, so it is no mask for a collective."""
     text = re.sub(r"//[^\n]*", "", open(path).read())
     assert "__activemask" not in text
+
+
+def test_shared_memory_limits_do_not_follow_the_call():
+    """A kernel's limit of dynamic shared memory is state that all threads
+    share: set to one call's size, it refuses the launch of another thread
+    whose blocks are larger.  One helper raises it, to a constant."""
+    uses = []
+    for path in glob.glob(os.path.join(CSRC, "*.cu*")):
+        text = re.sub(r"//[^\n]*", "", open(path).read())
+        uses += re.findall(r"cudaFuncSetAttribute\(([^;]*)\)", text)
+    assert len(uses) == 1 and re.sub(r"\s+", " ", uses[0]).endswith(
+        "cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_LIMIT")
