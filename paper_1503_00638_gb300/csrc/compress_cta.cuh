@@ -175,7 +175,7 @@ BSG_D void cta_gather_samples(const CodecArgs &a, uint8_t *buf, uint32_t c0, uin
     const uint2 *src = reinterpret_cast<const uint2 *>(a.in);
     uint2 *d = reinterpret_cast<uint2 *>(buf);
     const uint32_t tid = threadIdx.x, NT = blockDim.x;
-    if (2u * P.T > n) {
+    if (cta_gather_single(P.T, n)) {
 #pragma unroll 1
         for (uint32_t k = tid; k < n; k += NT) {
             const uint32_t c = c0 + k, s = fastdiv(c, P.dT), t = c - s * P.T;

@@ -28,6 +28,10 @@ __host__ __device__ constexpr bool cta_shape_ok(uint32_t es, uint32_t B)
            (es == 1 ? B % 128u == 0 : es == 2 ? B % 64u == 0 : B % 32u == 0);
 }
 
+// Whether the n samples of a block of a time-slowest cube are gathered one by
+// one: its time axis is longer than half the block (any length up to 2^32 - 1).
+__host__ __device__ constexpr bool cta_gather_single(uint32_t T, uint32_t n) { return T > n / 2u; }
+
 // Threads that hold a part of a block of Bb elements (whole groups, the last
 // one perhaps partial).
 template <int ES>
