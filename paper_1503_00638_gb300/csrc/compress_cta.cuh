@@ -23,8 +23,14 @@ enum CtaMode {
 // registers a thread.
 constexpr uint32_t CTA_WARPS_PER_SM = 28;
 
-// Full blocks from which a stream with a shortened last block takes two launches.
-constexpr uint32_t CTA_SPLIT_BLOCKS = 4096;
+// Bytes of full blocks of S bytes from which a stream with a shortened last
+// block takes two launches: what the fixed block size saves grows with the
+// stream, the second launch takes 5 to 8 us.  Walks, all in one launch and in
+// two: 64 MiB of 4-byte elements in 2, 4 and 8 KiB blocks 122, 77 and 73 us, and
+// 118, 80 and 74 (32 MiB 71, 47 and 46, and 74, 55 and 52; 128 MiB 224, 134 and
+// 128, and 205, 127 and 119); 64 MiB in 16 and 32 KiB 68 and 72, and 74 and 79,
+// 128 MiB 121 and 126, and 118 and 124.
+constexpr uint64_t cta_split_bytes(uint32_t S) { return (S <= 8192u ? 64ull : 128ull) << 20; }
 
 struct CtaPlan {
     uint32_t W;          // warps
@@ -562,7 +568,7 @@ cudaError_t launch_cta_order(const CodecArgs &a0, uint32_t max_ctas, cudaStream_
     const uint32_t nfull = a.nb - (a.last_B != a.B ? 1u : 0u);
     a.tile_begin = 0;
     a.tile_end = a.nb;
-    if (sizeof...(BCS) != 0 && (nfull == a.nb || nfull > CTA_SPLIT_BLOCKS)) {
+    if (sizeof...(BCS) != 0 && (nfull == a.nb || (uint64_t)nfull * a.B * ES >= cta_split_bytes(a.B * ES))) {
         cudaError_t e = cudaErrorNotReady;   // no such kernel
         a.tile_end = nfull;
         ((a.B == BCS ? (void)(e = launch_cta<LEVEL, ES, MODE, BCS, TS>(a, max_ctas, s)) : (void)0), ...);
