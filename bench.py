@@ -240,8 +240,9 @@ def run_reference(args, rank):
 # -- traffic recorded from an ncu capture of the current kernel source ----------
 
 # the sources the profiled compress kernel is compiled from
-KERNEL_SOURCES = ("kernels.cu", "kernels.cuh", "compress_cta.cuh", "lz4_cta.cuh",
-                  "shuffle_cta.cuh", "codec.cuh", "common.cuh",
+KERNEL_SOURCES = ("kernels.cu", "kernels.cuh", "compress_cta.cu", "compress_cta12.cu",
+                  "compress_cta8.cu", "compress_cta_vis.cu", "compress_cta_visx.cu",
+                  "compress_cta.cuh", "lz4_cta.cuh", "shuffle_cta.cuh", "codec.cuh", "common.cuh",
                   "lz4_warp.cuh", "shuffle.cuh")
 
 

@@ -491,10 +491,9 @@ BSG_D void compress_place(const CodecArgs &a, uint32_t tile, const uint8_t *blk,
 // this the streaming traffic evicts the dirty slot lines to DRAM for
 // nothing (measured on a 64-chunk batch: the compress launch's DRAM writes
 // 611 -> 393 MB for a 231 MB stream, 1008 -> 960 us).  The single-stream
-// fast kernel does not use it: its slots stay in L2 (its DRAM writes match
-// its stream) and the extra instructions cost it 2 %.  Only lines wholly inside [p, p + bytes) go (the lines at the
-// ends may hold a neighbouring slot); the caller has synchronised the warp
-// after its reads of the slot.
+// compressor does not use it: its slots stay in L2.  Only lines wholly inside
+// [p, p + bytes) go (the lines at the ends may hold a neighbouring slot); the
+// caller has synchronised the warp after its reads of the slot.
 BSG_D void discard_slot(const uint8_t *p, uint32_t bytes, uint32_t lane)
 {
     const uintptr_t a0 = ((uintptr_t)p + 127u) & ~(uintptr_t)127u;
@@ -572,67 +571,47 @@ struct FastPlan {
 static_assert(FAST_SLOT_BYTES >= r16(4 + lz4b(8192) + 32), "staging slot too small");
 
 // Round the 32 components of one group (16 samples t0 .. t0 + 15 of one
-// product) held as a[m] = component (m + 4 rot) mod 32.  GEN: int32 data or a
-// per-sample compensated c; otherwise float32 with the constant c, which is
-// kept as its own instantiation so that the common case carries no per-value
-// selects.
-template <bool GEN>
+// product) held as a[m] = component (m + 4 rot) mod 32: int32 data, a per-sample
+// compensated c or the constant one (float32 data with the constant c have
+// cta_round_group).
 BSG_D void round_group(const VisParams &P, uint32_t (&a)[32], uint32_t rot, uint32_t f,
                        uint32_t t0, const float *ai, const float *aj, bool is_auto)
 {
-    if (GEN) {
-        // c per sample: the compensated table (two adjacent samples per
-        // 8-byte load) or the constant; the data type is one branch per group
-        const float *crow = P.cft ? P.cft + (size_t)f * P.T + t0 : nullptr;
-        const float mul = is_auto ? 2.0f : 1.0f;  // exact: c2 = 2 c
-        auto qs = [&](uint32_t c, float &q0, float &q1) {
-            const float2 Ai = __ldg(reinterpret_cast<const float2 *>(ai + 2 * c));
-            const float2 Aj = __ldg(reinterpret_cast<const float2 *>(aj + 2 * c));
-            const float2 cc = crow ? __ldg(reinterpret_cast<const float2 *>(crow + 2 * c))
-                                   : make_float2(P.c, P.c);
-            q0 = __fmul_rn(__fmul_rn(__fmul_rn(cc.x, mul), Ai.x), Aj.x);
-            q1 = __fmul_rn(__fmul_rn(__fmul_rn(cc.y, mul), Ai.y), Aj.y);
-        };
-        if (P.is_int) {
-#pragma unroll
-            for (int k = 0; k < 8; k++) {
-                float q0, q1;
-                qs((k + rot) & 7u, q0, q1);
-                a[4 * k] = reduce_bits(a[4 * k], q0, true);
-                a[4 * k + 2] = reduce_bits(a[4 * k + 2], q1, true);
-                if (!is_auto) {
-                    a[4 * k + 1] = reduce_bits(a[4 * k + 1], q0, true);
-                    a[4 * k + 3] = reduce_bits(a[4 * k + 3], q1, true);
-                }
-            }
-        } else {
-#pragma unroll
-            for (int k = 0; k < 8; k++) {
-                float q0, q1;
-                qs((k + rot) & 7u, q0, q1);
-                a[4 * k] = __float_as_uint(reduce_one(__uint_as_float(a[4 * k]), q0));
-                a[4 * k + 2] = __float_as_uint(reduce_one(__uint_as_float(a[4 * k + 2]), q1));
-                if (!is_auto) {
-                    a[4 * k + 1] = __float_as_uint(reduce_one(__uint_as_float(a[4 * k + 1]), q0));
-                    a[4 * k + 3] = __float_as_uint(reduce_one(__uint_as_float(a[4 * k + 3]), q1));
-                }
-            }
-        }
-        return;
-    }
-    const float cc = is_auto ? P.c2 : P.c;
-#pragma unroll
-    for (int k = 0; k < 8; k++) {
-        const uint32_t c = (k + rot) & 7u;  // chunk c: samples t0 + 2c, t0 + 2c + 1
+    // c per sample: the compensated table (two adjacent samples per
+    // 8-byte load) or the constant; the data type is one branch per group
+    const float *crow = P.cft ? P.cft + (size_t)f * P.T + t0 : nullptr;
+    const float mul = is_auto ? 2.0f : 1.0f;  // exact: c2 = 2 c
+    auto qs = [&](uint32_t c, float &q0, float &q1) {
         const float2 Ai = __ldg(reinterpret_cast<const float2 *>(ai + 2 * c));
         const float2 Aj = __ldg(reinterpret_cast<const float2 *>(aj + 2 * c));
-        const float q0 = __fmul_rn(__fmul_rn(cc, Ai.x), Aj.x);
-        const float q1 = __fmul_rn(__fmul_rn(cc, Ai.y), Aj.y);
-        a[4 * k] = __float_as_uint(reduce_one(__uint_as_float(a[4 * k]), q0));
-        a[4 * k + 2] = __float_as_uint(reduce_one(__uint_as_float(a[4 * k + 2]), q1));
-        if (!is_auto) {
-            a[4 * k + 1] = __float_as_uint(reduce_one(__uint_as_float(a[4 * k + 1]), q0));
-            a[4 * k + 3] = __float_as_uint(reduce_one(__uint_as_float(a[4 * k + 3]), q1));
+        const float2 cc = crow ? __ldg(reinterpret_cast<const float2 *>(crow + 2 * c))
+                               : make_float2(P.c, P.c);
+        q0 = __fmul_rn(__fmul_rn(__fmul_rn(cc.x, mul), Ai.x), Aj.x);
+        q1 = __fmul_rn(__fmul_rn(__fmul_rn(cc.y, mul), Ai.y), Aj.y);
+    };
+    if (P.is_int) {
+#pragma unroll
+        for (int k = 0; k < 8; k++) {
+            float q0, q1;
+            qs((k + rot) & 7u, q0, q1);
+            a[4 * k] = reduce_bits(a[4 * k], q0, true);
+            a[4 * k + 2] = reduce_bits(a[4 * k + 2], q1, true);
+            if (!is_auto) {
+                a[4 * k + 1] = reduce_bits(a[4 * k + 1], q0, true);
+                a[4 * k + 3] = reduce_bits(a[4 * k + 3], q1, true);
+            }
+        }
+    } else {
+#pragma unroll
+        for (int k = 0; k < 8; k++) {
+            float q0, q1;
+            qs((k + rot) & 7u, q0, q1);
+            a[4 * k] = __float_as_uint(reduce_one(__uint_as_float(a[4 * k]), q0));
+            a[4 * k + 2] = __float_as_uint(reduce_one(__uint_as_float(a[4 * k + 2]), q1));
+            if (!is_auto) {
+                a[4 * k + 1] = __float_as_uint(reduce_one(__uint_as_float(a[4 * k + 1]), q0));
+                a[4 * k + 3] = __float_as_uint(reduce_one(__uint_as_float(a[4 * k + 3]), q1));
+            }
         }
     }
 }
@@ -659,7 +638,6 @@ BSG_D void round_group_full(const VisParams &P, uint32_t (&a)[32], uint32_t rot,
     }
 }
 
-template <bool GEN>
 struct VisGroupRound {
     const VisParams *P;
     uint32_t c_blk;  // complex index of the block's first sample
@@ -674,7 +652,7 @@ struct VisGroupRound {
         const uint32_t ij = __ldg(P->pairs + p);
         const uint32_t i = ij & 0xffffu, j = ij >> 16;
         const bool is_auto = i == j;
-        if (GEN && P->qtab) {
+        if (P->qtab) {
             // full covariance: the q rows of the Re and Im components ([F][M][T])
             const float *qre = P->qtab + ((size_t)f * P->M + p) * P->T + t0;
             const float *qim = P->qtab + ((size_t)f * P->M + P->P + p - i - 1) * P->T + t0;
@@ -683,7 +661,7 @@ struct VisGroupRound {
         }
         const float *ai = P->autos + (size_t)(f * P->n_in + i) * P->T + t0;
         const float *aj = P->autos + (size_t)(f * P->n_in + j) * P->T + t0;
-        round_group<GEN>(*P, a, rot, f, t0, ai, aj, is_auto);
+        round_group(*P, a, rot, f, t0, ai, aj, is_auto);
     }
 };
 

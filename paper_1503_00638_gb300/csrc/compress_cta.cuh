@@ -19,8 +19,9 @@ enum CtaMode {
     CTA_SAMPLE    // any time axis and 8-byte samples: in shared memory first
 };
 
-// Resident warps per SM of the kernels with a fixed block size: 28 at 72
-// registers a thread.
+// Resident warps per SM of the kernels with a fixed block size of one or two
+// warps: 28, with 72 registers a thread.  Larger blocks have 32 at 64 (a CTA more
+// per SM counts for more there), as the kernel of any size.
 constexpr uint32_t CTA_WARPS_PER_SM = 28;
 
 // Bytes of full blocks of S bytes from which a stream with a shortened last
@@ -123,7 +124,7 @@ struct CtaRound {
     BSG_D void operator()(uint32_t g, uint32_t (&v)[32]) const
     {
         if (MODE == CTA_GROUP_X) {
-            const VisGroupRound<true> round{P, c_blk};
+            const VisGroupRound round{P, c_blk};
             round(g, v);
         } else if (MODE == CTA_GROUP) {
             const uint32_t cg = c_blk + 16u * g;

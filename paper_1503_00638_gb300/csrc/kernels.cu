@@ -615,13 +615,11 @@ __global__ void compress_small_kernel(const __grid_constant__ CodecArgs a)
     if (lane == 0) *a.out_bytes = 12 + tb;
 }
 
-// One warp per CTA, persistent.  Per block: wait for its stream bytes in
-// `comp`, LZ4-decode into `dec`, start the next block's copy into `comp`,
-// un-transpose `dec` in place and bulk-store it (blocks the register paths
-// cannot take are un-transposed into `comp` and stored before the next copy).
-// ES: 4 or 8 compiles the in-place register un-transpose for that element
-// size; 0 compiles only the general path.
-template <uint32_t MAXB, int ES>
+// The general decoder (block sizes whose blocks are not 16-byte aligned in the
+// output).  One warp per CTA, persistent.  Per block: wait for its stream bytes
+// in `comp`, LZ4-decode into `dec`, un-transpose into `comp` and store, then start
+// the next block's copy into `comp`.
+template <uint32_t MAXB>
 __global__ void __launch_bounds__(32, MAXB <= 8192 ? 13 : 1)
     decompress_kernel(const __grid_constant__ CodecArgs a)
 {
@@ -660,9 +658,6 @@ __global__ void __launch_bounds__(32, MAXB <= 8192 ? 13 : 1)
         const uint32_t Bb = block_elems_of(a, tile);
         const uint32_t S = Bb * a.es;
         const uint32_t nxt = grab_tile(a.tile_counter, lane);
-        // the previous block's bulk store must have finished reading `dec`
-        if (lane == 0) bulk_wait_read0();
-        __syncwarp();
         bool good = cur.ok;
         if (good) {
             if (cur.eidx != ~0u) comp[cur.eidx] = cur.ebyte;
@@ -672,8 +667,7 @@ __global__ void __launch_bounds__(32, MAXB <= 8192 ? 13 : 1)
         }
         if (!good && lane == 0) set_status(a.status, BSGPU_ERR_CORRUPT);
         uint8_t *dst = a.out + (uint64_t)tile * a.B * a.es;
-        const bool inplace = ES != 0 && MAXB <= 8192 && unshuffle_inplace_ok(a.es, Bb);
-        if (good && !inplace) {
+        if (good) {
             unshuffle_block(dec, comp, Bb, a.es, lane);
             __syncwarp();
             for (uint32_t k = lane; k < S; k += 32) dst[k] = comp[k];
@@ -687,25 +681,6 @@ __global__ void __launch_bounds__(32, MAXB <= 8192 ? 13 : 1)
             __syncwarp();
             ld = dec_issue(a, nxt, comp, bar, lane);
         }
-        if (good && inplace) {
-            if (ES == 2)
-                unshuffle2_inplace(dec, Bb, lane);
-            else if (ES == 4)
-                unshuffle4_inplace(dec, Bb, lane);
-            else if (ES == 8)
-                unshuffle8_inplace(dec, Bb, lane);
-            __syncwarp();
-            if ((S & 15u) == 0 && ((uintptr_t)dst & 15u) == 0) {
-                fence_proxy_async_smem();
-                __syncwarp();
-                if (lane == 0) {
-                    bulk_s2g(dst, dec, S);
-                    bulk_commit();
-                }
-            } else {
-                for (uint32_t k = lane; k < S; k += 32) dst[k] = dec[k];
-            }
-        }
         if (tile + 1 == a.nb) {
             const uint32_t tb = a.tail_elems * a.es;
             const uint64_t first = (a.n_elem - a.tail_elems) * a.es;
@@ -716,8 +691,6 @@ __global__ void __launch_bounds__(32, MAXB <= 8192 ? 13 : 1)
         __syncwarp();
         tile = nxt;
     }
-    if (lane == 0) bulk_wait0();
-    __syncwarp();
 }
 
 // Decompress with ONE shared buffer per warp, for blocks of at most 8 KiB whose
@@ -1674,15 +1647,10 @@ cudaError_t launch_decompress(const CodecArgs &a, uint32_t maxb, uint32_t grid, 
         if (a.es == 4) return launch_warp_kernel(decompress_inplace_kernel<4>, sm1, grid, s, a);
         return launch_warp_kernel(decompress_inplace_kernel<8>, sm1, grid, s, a);
     }
-    if (maxb <= 8192) {
-        if (a.es == 2) return launch_warp_kernel(decompress_kernel<8192, 2>, smem, grid, s, a);
-        if (a.es == 4) return launch_warp_kernel(decompress_kernel<8192, 4>, smem, grid, s, a);
-        if (a.es == 8) return launch_warp_kernel(decompress_kernel<8192, 8>, smem, grid, s, a);
-        return launch_warp_kernel(decompress_kernel<8192, 0>, smem, grid, s, a);
-    }
-    if (maxb <= 16384) return launch_warp_kernel(decompress_kernel<16384, 0>, smem, grid, s, a);
-    if (maxb <= 32768) return launch_warp_kernel(decompress_kernel<32768, 0>, smem, grid, s, a);
-    return launch_warp_kernel(decompress_kernel<65536, 0>, smem, grid, s, a);
+    if (maxb <= 8192) return launch_warp_kernel(decompress_kernel<8192>, smem, grid, s, a);
+    if (maxb <= 16384) return launch_warp_kernel(decompress_kernel<16384>, smem, grid, s, a);
+    if (maxb <= 32768) return launch_warp_kernel(decompress_kernel<32768>, smem, grid, s, a);
+    return launch_warp_kernel(decompress_kernel<65536>, smem, grid, s, a);
 }
 
 cudaError_t launch_decompress_inplace_any(const CodecArgs &a, uint32_t maxb, uint32_t grid, cudaStream_t s)

@@ -6,9 +6,9 @@
 // Why a CTA and not a warp: the block is the unit that shared memory holds,
 // so one warp per block leaves an SM with as many warps as blocks fit (20 at
 // 8 KiB, 3 at 64 KiB) and the encoder bound by the latency of one warp's
-// serial steps.  Here a block of S bytes gets a thread per 128 bytes: 32
-// warps per SM at 64 registers for every block size, each thread holding one
-// 32-word group of the bit transpose.
+// serial steps.  Here a block of S bytes gets a thread per 128 bytes: 28 to 32
+// warps per SM for every block size, each thread holding one 32-word group of
+// the bit transpose.
 //
 // The stages of level 0, a barrier between each:
 //   1. word-equality bitmaps E[k] = {row, run} (the caller, or
@@ -183,7 +183,7 @@ BSG_D uint32_t cta_first_set(const CtaScratch &c, uint32_t from, uint32_t to, ui
 }
 
 // Encode src[0, S) (shared, word aligned, readable to S + 8; S a multiple of
-// 8, at most 4096 W) into dst (4 bytes past a 16-byte boundary, capacity
+// 8, at most 4096 W at level 0 and 8192 W at level 1) into dst (4 bytes past a 16-byte boundary, capacity
 // lz4_bound(S)); c.E
 // holds the block's bitmaps, a barrier passed since they were written.
 // size_known(cs) is called by every thread as soon as the size is known,
